@@ -23,6 +23,8 @@ namespace {
 constexpr int kNumLayers = 10;
 constexpr int kLossBlocks = 1024;
 constexpr int kStatBlocks = 256;
+static_assert(kFields * kStatBlocks * 2 >= kShiftPartials,
+              "the warm start's mean shifts reuse the field statistics' scratch");
 
 struct Layer {
   // definition
@@ -697,7 +699,7 @@ int mclbm_net_forward(mclbm_net_t* n, int batch, const float* cond, float* field
   cudaError_t e = forward(n, batch, cond);
   if (e == cudaSuccess)
     e = launch_denormalize(n->L[kNumLayers - 1].pre, n->norm, cond, batch,
-                           n->cfg.ny * n->cfg.nx, fields, n->stream);
+                           n->cfg.ny * n->cfg.nx, n->stat_part, fields, n->stream);
   return e == cudaSuccess ? MCLBM_OK : cuda_fail(n, e, "mclbm_net_forward");
 }
 

@@ -185,8 +185,10 @@ cudaError_t launch_uniform_fill(float* p, int64_t n, float scale, uint64_t seed,
 cudaError_t launch_geometry(float* X, int batch, int ny, int nx, cudaStream_t st);
 // fields[b][ch][i] = base[b][ch] + mean[ch] + scale[ch] * out[ch][b*hw + i]; phi (ch 3) and
 // rho^w (ch 4) are then shifted so that their means are phi_0 = cond[b][1] and 1 - phi_0.
+// partial: kShiftPartials doubles of scratch (batch <= 256: at least five chunks per sample).
+constexpr int kShiftPartials = 2560;
 cudaError_t launch_denormalize(const float* out, const float* norm, const float* cond, int batch,
-                               int hw, float* fields, cudaStream_t st);
+                               int hw, double* partial, float* fields, cudaStream_t st);
 // Per-channel FP64 sum and sum of squares of fields - base, fields [n][5][hw], cond [n][3], into
 // partial[5][blocks][2].
 cudaError_t launch_field_moments(const float* fields, const float* cond, int n, int hw,
