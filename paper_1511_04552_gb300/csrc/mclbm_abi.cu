@@ -431,7 +431,7 @@ int mclbm_nusselt(mclbm_t* h, double* nu_hot, double* nu_cold) {
   int rc = ready(h, true);
   if (rc) return rc;
   if (!nu_hot || !nu_cold) return fail(h, MCLBM_EINVAL, "NULL output");
-  CK(h, launch_nusselt(h->state[h->cur], h->L, h->k, h->red, h->stream));
+  CK(h, launch_nusselt(h->state[h->cur], h->L, h->k, h->partials, h->red, h->stream));
   double s[2];
   rc = d2h_sync(h, s, h->red, sizeof(s));
   if (rc) return rc;
@@ -476,7 +476,7 @@ int mclbm_diagnostics(mclbm_t* h, double* nu_hot, double* nu_cold, double* mass_
   // the three reductions one after another on the stream, each into its own slot of the
   // result area (the partial sums are reused in stream order), then one copy and one wait
   const int64_t K = h->steps - h->snap_steps;
-  CK(h, launch_nusselt(h->state[h->cur], h->L, h->k, h->red, h->stream));
+  CK(h, launch_nusselt(h->state[h->cur], h->L, h->k, h->partials, h->red, h->stream));
   CK(h, launch_mass(h->state[h->cur], h->L, h->partials, h->red + kRedWidth, h->stream));
   CK(h, launch_residual(h->state[h->cur], h->L, h->k, h->snap, K > 0, h->partials,
                         h->red + 2 * kRedWidth, h->stream));

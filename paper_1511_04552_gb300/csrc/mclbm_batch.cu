@@ -58,28 +58,13 @@ __global__ void __launch_bounds__(pair::Threads<2, kBatchTileW>::value,
 
 // Nusselt sums of every cavity: block c reduces cavity c (the same sums as nusselt_kernel).
 template <class T>
-__global__ void batch_nusselt_kernel(const BatchCav* __restrict__ cavs, int parity,
+__global__ void __launch_bounds__(kWallThreads) batch_nusselt_kernel(const BatchCav* __restrict__ cavs, int parity,
                                      double* __restrict__ out) {
   const BatchCav& cv = cavs[blockIdx.x];
-  const Layout L = cv.L;
-  const T* src = static_cast<const T*>(cv.level[cv.cur ^ parity]);
-  const float s = cv.k.inv_nx;
   double acc[2] = {0.0, 0.0};
-  for (int j = threadIdx.x; j < L.ny; j += blockDim.x) {
-    float fw[kQ], fp[kQ], g[kQ];
-    pull_node<T, false>(src, L, 0, j, fw, fp, g, s);
-    const double t0 = sum9(g);
-    pull_node<T, false>(src, L, 1, j, fw, fp, g, s);
-    const double t1 = sum9(g);
-    pull_node<T, false>(src, L, L.nx - 1, j, fw, fp, g, s);
-    const double c0 = sum9(g);
-    pull_node<T, false>(src, L, L.nx - 2, j, fw, fp, g, s);
-    const double c1 = sum9(g);
-    const double slope = 1.0 / (double)L.nx;
-    acc[0] += slope + (t1 - 9.0 * t0) / 3.0;
-    acc[1] += slope + (9.0 * c0 - c1) / 3.0;
-  }
-  __shared__ double sm[8][2];
+  wall_gradients<T>(static_cast<const T*>(cv.level[cv.cur ^ parity]), cv.L, cv.k, 0, kWallRows,
+                    acc);
+  __shared__ double sm[kWallThreads / 32][2];
   for (int c = 0; c < 2; ++c)
     for (int off = 16; off > 0; off >>= 1) acc[c] += __shfl_down_sync(0xffffffffu, acc[c], off);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -165,14 +150,14 @@ cudaError_t launch_batch_nusselt(const BatchLaunch& b, int n_cav, int parity, do
                                  cudaStream_t st) {
   switch (b.storage) {
     case MCLBM_STORE_F32:
-      batch_nusselt_kernel<float><<<n_cav, 256, 0, st>>>((const BatchCav*)b.cavs, parity, out);
+      batch_nusselt_kernel<float><<<n_cav, kWallThreads, 0, st>>>((const BatchCav*)b.cavs, parity, out);
       break;
     case MCLBM_STORE_F16:
-      batch_nusselt_kernel<__half><<<n_cav, 256, 0, st>>>((const BatchCav*)b.cavs, parity, out);
+      batch_nusselt_kernel<__half><<<n_cav, kWallThreads, 0, st>>>((const BatchCav*)b.cavs, parity, out);
       break;
     case MCLBM_STORE_BF16:
       batch_nusselt_kernel<__nv_bfloat16>
-          <<<n_cav, 256, 0, st>>>((const BatchCav*)b.cavs, parity, out);
+          <<<n_cav, kWallThreads, 0, st>>>((const BatchCav*)b.cavs, parity, out);
       break;
     default:
       return cudaErrorInvalidValue;

@@ -227,6 +227,47 @@ __device__ __forceinline__ Moments moments_of(const float* fw, const float* fp, 
   return m;
 }
 
+// The (mixture) temperature's deviation from theta_c at node (i, j) after streaming.
+template <class T>
+__device__ __forceinline__ float node_theta_dev(const T* __restrict__ src, const Layout& L,
+                                                const StepConsts& k, int i, int j) {
+  const float s = k.inv_nx;
+  float fw[kQ], fp[kQ], g[kQ];
+  if (!k.two_sets) {
+    pull_node<T, false>(src, L, i, j, fw, fp, g, s);
+    return sum9(g);
+  }
+  pull_node<T, true>(src, L, i, j, fw, fp, g, s);
+  const float dw = sum9(g);
+  pull_thermal<T>(src, L, i, j, 3 * kQ, g, s);
+  return mixture_dev(k, k.rho_w0 + sum9(fw), k.rho_p0 + sum9(fp), dw, sum9(g));
+}
+
+// Wall gradients from the theta deviations (the Eq 33 mixture's with two sets): with
+// theta = theta_c + theta', (8 T_h - 9 theta_0 + theta_1)/3 = 1/nx + (theta'_1 - 9 theta'_0)/3
+// and the cold-wall twin (9 theta_{n-1} - theta_{n-2} - 8 T_c)/3
+// = 1/nx + (9 theta'_{n-1} - theta'_{n-2})/3. Adds the rows j0, j0 + step, ... to acc (hot,
+// cold). Four threads share a row, one per node it needs: the pulls are chains of dependent
+// cache misses, so a thread that did all four of them spent its time waiting.
+template <class T>
+__device__ __forceinline__ void wall_gradients(const T* __restrict__ src, const Layout& L,
+                                               const StepConsts& k, int j0, int step,
+                                               double (&acc)[2]) {
+  const int col = threadIdx.x & 3;
+  const int i = col < 2 ? col : L.nx + 1 - col;
+  const double slope = 1.0 / (double)L.nx;
+  for (int jb = j0; jb < L.ny; jb += step) {  // the same trips for every thread of a block
+    const int j = jb + (int)(threadIdx.x >> 2);
+    const bool in = j < L.ny;
+    const double own = in ? (double)node_theta_dev(src, L, k, i, j) : 0.0;
+    const double next = __shfl_down_sync(0xffffffffu, own, 1);
+    if (in && col == 0) acc[0] += slope + (next - 9.0 * own) / 3.0;
+    if (in && col == 2) acc[1] += slope + (9.0 * own - next) / 3.0;
+  }
+}
+constexpr int kWallThreads = 512;           // 128 rows at a time
+constexpr int kWallRows = kWallThreads / 4;
+
 // Per-step hash that seeds the rounding streams: the launch's seed and the graph epoch.
 __device__ __forceinline__ uint32_t step_hash(const StepArgs& a) {
   const uint32_t ep = a.epoch ? *(volatile const uint32_t*)a.epoch : 0u;

@@ -126,8 +126,9 @@ cudaError_t launch_init(void* dst, const Layout& L, const StepConsts& k, const f
 cudaError_t launch_fields(const void* src, const Layout& L, const StepConsts& k, uint32_t which,
                           float* out, cudaStream_t st);
 // Nusselt partial sums: red[0] = sum_j (8 T_h - 9 th_0 + th_1) / 3, red[1] = cold-wall twin.
-cudaError_t launch_nusselt(const void* src, const Layout& L, const StepConsts& k, double* red,
-                           cudaStream_t st);
+// partials: scratch of kMaxRedBlocks x kRedWidth doubles, as for the other reductions.
+cudaError_t launch_nusselt(const void* src, const Layout& L, const StepConsts& k,
+                           double* partials, double* red, cudaStream_t st);
 // Mass: red[0] = sum of f^w deviations, red[1] = sum of f^p deviations.
 cudaError_t launch_mass(const void* src, const Layout& L, double* partials, double* red,
                         cudaStream_t st);

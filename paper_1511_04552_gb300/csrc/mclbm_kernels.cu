@@ -158,37 +158,45 @@ __global__ void final_reduce_kernel(const double* __restrict__ partials, int cou
   block_reduce_store<kRedWidth>(acc, red);
 }
 
-// Wall gradients from the theta deviations (the Eq 33 mixture's with two sets): with
-// theta = theta_c + theta', (8 T_h - 9 theta_0 + theta_1)/3 = 1/nx + (theta'_1 - 9 theta'_0)/3
-// and the cold-wall twin (9 theta_{n-1} - theta_{n-2} - 8 T_c)/3
-// = 1/nx + (9 theta'_{n-1} - theta'_{n-2})/3.
+// Wall sums of rows blockIdx.x kWallRows, + gridDim.x kWallRows, ... into out + blockIdx.x stride.
+// Latency-bound (4 nodes per row): with one block of 256 threads and four pulls per thread a
+// 1024-row cavity took 60 us; eight blocks take 13 us and their final sum 8 us.
 template <class T>
-__global__ void nusselt_kernel(const T* __restrict__ src, const Layout L, const StepConsts k,
-                               double* __restrict__ red) {
-  const float s = k.inv_nx;
-  // the (mixture) temperature's deviation from theta_c at node (i, j) after streaming
-  auto dev = [&](int i, int j) -> float {
-    float fw[kQ], fp[kQ], g[kQ];
-    if (!k.two_sets) {
-      pull_node<T, false>(src, L, i, j, fw, fp, g, s);
-      return sum9(g);
-    }
-    pull_node<T, true>(src, L, i, j, fw, fp, g, s);
-    const float dw = sum9(g);
-    pull_thermal<T>(src, L, i, j, 3 * kQ, g, s);
-    return mixture_dev(k, k.rho_w0 + sum9(fw), k.rho_p0 + sum9(fp), dw, sum9(g));
-  };
-  double acc[2] = {0.0, 0.0};
-  for (int j = threadIdx.x; j < L.ny; j += blockDim.x) {
-    const double t0 = dev(0, j);
-    const double t1 = dev(1, j);
-    const double c0 = dev(L.nx - 1, j);
-    const double c1 = dev(L.nx - 2, j);
-    const double slope = 1.0 / (double)L.nx;
-    acc[0] += slope + (t1 - 9.0 * t0) / 3.0;
-    acc[1] += slope + (9.0 * c0 - c1) / 3.0;
-  }
-  block_reduce_store<2>(acc, red);
+__global__ void __launch_bounds__(kWallThreads)
+    nusselt_kernel(const T* __restrict__ src, const Layout L, const StepConsts k,
+                   double* __restrict__ out) {
+  double acc[kRedWidth];
+#pragma unroll
+  for (int c = 0; c < kRedWidth; ++c) acc[c] = 0.0;
+  double wall[2] = {0.0, 0.0};
+  wall_gradients<T>(src, L, k, (int)blockIdx.x * kWallRows, (int)gridDim.x * kWallRows, wall);
+  acc[0] = wall[0];
+  acc[1] = wall[1];
+  block_reduce_store<kRedWidth>(acc, out + (size_t)blockIdx.x * kRedWidth);
+}
+
+// a + b = s + e exactly (Knuth's two-sum; no operation below can be contracted)
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
+  return s;
+}
+
+// Adds nine stored populations of a node to an FP64 sum. GB300 does 2 FP64 operations per clock
+// and SM against 128 in FP32, and nine conversions with nine additions per node and component
+// were what the mass reduction waited for; so the nine are first summed in FP32 with the exact
+// errors of the additions kept beside the sum (a tree of two-sums: s + e is the exact sum to
+// about 2^-45 of the terms), and the two parts go to the FP64 sum. 1024 x 1024: 78 us before,
+// 30 us now.
+__device__ __forceinline__ void add_nine(const float (&v)[kQ], double& acc) {
+  float e[8];
+  const float a = two_sum(v[0], v[1], e[0]), b = two_sum(v[2], v[3], e[1]);
+  const float c = two_sum(v[4], v[5], e[2]), d = two_sum(v[6], v[7], e[3]);
+  const float ab = two_sum(a, b, e[4]), cd = two_sum(c, d, e[5]);
+  const float abcd = two_sum(ab, cd, e[6]);
+  const float s = two_sum(abcd, v[8], e[7]);
+  acc += (double)s;
+  acc += (double)(((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7])));
 }
 
 template <class T>
@@ -202,11 +210,14 @@ __global__ void mass_kernel(const T* __restrict__ src, const Layout L,
        t += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(t % L.nx), j = (int)(t / L.nx);
     const size_t o = (size_t)j * L.pitch + i;
+    float fw[kQ], fp[kQ];
 #pragma unroll
     for (int q = 0; q < kQ; ++q) {
-      acc[0] += (double)Elem<T>::ldg(src + (size_t)q * L.plane + o);
-      acc[1] += (double)Elem<T>::ldg(src + (size_t)(kQ + q) * L.plane + o);
+      fw[q] = Elem<T>::ldg(src + (size_t)q * L.plane + o);
+      fp[q] = Elem<T>::ldg(src + (size_t)(kQ + q) * L.plane + o);
     }
+    add_nine(fw, acc[0]);
+    add_nine(fp, acc[1]);
   }
   block_reduce_store<kRedWidth>(acc, partials + (size_t)blockIdx.x * kRedWidth);
 }
@@ -250,20 +261,47 @@ __global__ void residual_kernel(const T* __restrict__ src, const Layout L, const
   if (sums) block_reduce_store<kRedWidth>(acc, partials + (size_t)blockIdx.x * kRedWidth);
 }
 
-template <class T>
+// One row of one plane per block: no division per element, and rows whose packed start is 16-byte
+// aligned (nx a multiple of 4) move four elements per thread. Bound by memory (read and write
+// once). 1024 x 1024 FP32, 226 MB: 88 us with a flat index and 64-bit divisions, now 38 us.
+template <class T, int V>
 __global__ void state_copy_kernel(const void* __restrict__ src_v, void* __restrict__ dst_v,
                                   const Layout L, int to_packed) {
   const int64_t n = (int64_t)L.nx * L.ny;
-  const int64_t total = n * L.np;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = t / n, r = t % n;
-    const int i = (int)(r % L.nx), j = (int)(r / L.nx);
-    const size_t po = (size_t)p * L.plane + (size_t)j * L.pitch + i;
-    if (to_packed)
-      static_cast<float*>(dst_v)[t] = Elem<T>::get(static_cast<const T*>(src_v)[po]);
-    else
-      static_cast<T*>(dst_v)[po] = Elem<T>::put(static_cast<const float*>(src_v)[t]);
+  const int64_t rows = (int64_t)L.np * L.ny;
+  const int per_row = blockDim.x, sub = threadIdx.y;  // blockDim.y rows side by side
+  for (int64_t r = blockIdx.x * (int64_t)blockDim.y + sub; r < rows;
+       r += (int64_t)gridDim.x * blockDim.y) {
+    const int p = (int)(r / L.ny), j = (int)(r % L.ny);
+    const size_t stored = (size_t)p * L.plane + (size_t)j * L.pitch;
+    const size_t packed = (size_t)p * n + (size_t)j * L.nx;
+    for (int i = threadIdx.x * V; i < L.nx; i += per_row * V) {
+      if constexpr (V == 1) {
+        if (to_packed)
+          static_cast<float*>(dst_v)[packed + i] =
+              Elem<T>::get(static_cast<const T*>(src_v)[stored + i]);
+        else
+          static_cast<T*>(dst_v)[stored + i] =
+              Elem<T>::put(static_cast<const float*>(src_v)[packed + i]);
+      } else {
+        struct alignas(4 * sizeof(T)) Quad { T v[4]; };
+        if (to_packed) {
+          const Quad q = *reinterpret_cast<const Quad*>(static_cast<const T*>(src_v) + stored + i);
+          *reinterpret_cast<float4*>(static_cast<float*>(dst_v) + packed + i) =
+              make_float4(Elem<T>::get(q.v[0]), Elem<T>::get(q.v[1]), Elem<T>::get(q.v[2]),
+                          Elem<T>::get(q.v[3]));
+        } else {
+          const float4 f = *reinterpret_cast<const float4*>(
+              static_cast<const float*>(src_v) + packed + i);
+          Quad q;
+          q.v[0] = Elem<T>::put(f.x);
+          q.v[1] = Elem<T>::put(f.y);
+          q.v[2] = Elem<T>::put(f.z);
+          q.v[3] = Elem<T>::put(f.w);
+          *reinterpret_cast<Quad*>(static_cast<T*>(dst_v) + stored + i) = q;
+        }
+      }
+    }
   }
 }
 
@@ -458,11 +496,16 @@ cudaError_t launch_fields(const void* src, const Layout& L, const StepConsts& k,
   });
 }
 
-cudaError_t launch_nusselt(const void* src, const Layout& L, const StepConsts& k, double* red,
-                           cudaStream_t st) {
+// Up to 2 kWallRows rows one block walks them and writes the result itself (a second launch
+// costs as much as a second trip); beyond, kWallRows rows per block and a final sum.
+cudaError_t launch_nusselt(const void* src, const Layout& L, const StepConsts& k,
+                           double* partials, double* red, cudaStream_t st) {
+  const int g = L.ny <= 2 * kWallRows ? 1 : grid_for(L.ny, kWallRows, kMaxRedBlocks);
   return by_storage(L.storage, [&](auto* tag) {
     using T = std::remove_pointer_t<decltype(tag)>;
-    nusselt_kernel<T><<<1, 256, 0, st>>>(static_cast<const T*>(src), L, k, red);
+    nusselt_kernel<T><<<g, kWallThreads, 0, st>>>(static_cast<const T*>(src), L, k,
+                                                  g == 1 ? red : partials);
+    if (g > 1) final_reduce_kernel<<<1, 256, 0, st>>>(partials, g, red);
     return cudaGetLastError();
   });
 }
@@ -482,7 +525,9 @@ cudaError_t launch_mass(const void* src, const Layout& L, double* partials, doub
 cudaError_t launch_residual(const void* src, const Layout& L, const StepConsts& k, float* snap,
                             bool sums, double* partials, double* red, cudaStream_t st) {
   const int64_t n = (int64_t)L.nx * L.ny;
-  const int g = grid_for(n, 256, kMaxRedBlocks);
+  // the sums want few blocks (their FP64 block reductions), a snapshot alone as many as it can
+  // get (1024 x 1024: 47 us with 304 blocks, 33 us with 4096)
+  const int g = grid_for(n, 256, sums ? kMaxRedBlocks : 4096);
   return by_storage(L.storage, [&](auto* tag) {
     using T = std::remove_pointer_t<decltype(tag)>;
     residual_kernel<T><<<g, 256, 0, st>>>(static_cast<const T*>(src), L, k, snap, sums ? 1 : 0,
@@ -492,12 +537,23 @@ cudaError_t launch_residual(const void* src, const Layout& L, const StepConsts& 
   });
 }
 
+// Four elements per thread where both sides of a row allow it: stored rows start on 128 bytes,
+// packed ones on nx floats, and the caller's array may start anywhere.
 cudaError_t launch_state_copy(const void* src, void* dst, const Layout& L, bool to_packed,
                               cudaStream_t st) {
-  const int64_t n = (int64_t)L.nx * L.ny * L.np;
+  const void* packed = to_packed ? dst : src;
+  const bool quads = L.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(packed) & 15u) == 0;
+  const int per_row = quads ? L.nx / 4 : L.nx;
+  const int bx = per_row <= 32 ? 32 : (per_row <= 64 ? 64 : (per_row <= 128 ? 128 : 256));
+  const dim3 block(bx, 256 / bx);
+  const int64_t rows = (int64_t)L.np * L.ny;
+  const int grid = grid_for(rows, (int)block.y, 1 << 16);
   return by_storage(L.storage, [&](auto* tag) {
     using T = std::remove_pointer_t<decltype(tag)>;
-    state_copy_kernel<T><<<grid_for(n, 256, 8192), 256, 0, st>>>(src, dst, L, to_packed ? 1 : 0);
+    if (quads)
+      state_copy_kernel<T, 4><<<grid, block, 0, st>>>(src, dst, L, to_packed ? 1 : 0);
+    else
+      state_copy_kernel<T, 1><<<grid, block, 0, st>>>(src, dst, L, to_packed ? 1 : 0);
     return cudaGetLastError();
   });
 }
