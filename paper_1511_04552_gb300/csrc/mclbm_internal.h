@@ -47,6 +47,8 @@ struct StepConsts {
   float r_cp;                 // C_p,p / C_p,f: the heat-capacity weight of Eq 33
   double rho_w0_d, rho_p0_d;  // FP64 offsets and rho_f / rho_p for the initial fill
   double fr_d;
+  double inv_fr_d, inv_nx_d;   // 1 / fr_d and 1 / nx for the initial fill
+  float inv_fr_h, inv_fr_l;    // 1 / fr_d as a sum of two FP32 numbers
 };
 
 // Layout of the state inside the caller's buffer: np planes [ny][pitch] per time level.

@@ -39,43 +39,159 @@ __global__ void stream_only_kernel(const T* __restrict__ src, T* __restrict__ ds
   }
 }
 
+// a + b = s + e exactly (Knuth's two-sum; no operation below can be contracted)
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
+  return s;
+}
+
 // ---- initial equilibrium (Eqs 26-27) ---------------------------------------------------------
+// One node in FP64 from the caller's fields, so that the stored values are correctly rounded.
 template <class T>
-__global__ void init_kernel(T* __restrict__ dst, const Layout L, const StepConsts k,
-                            const float* __restrict__ warm, int warm_rho) {
-  const int64_t n = (int64_t)L.nx * L.ny;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(t % L.nx), j = (int)(t / L.nx);
-    // FP64 here (once per run) so that the stored values are correctly rounded
-    double ux = 0.0, uy = 0.0, th, drw = 0.0, drp = 0.0;
-    if (warm) {
-      ux = warm[t];
-      uy = warm[n + t];
-      th = warm[2 * n + t];
-      const double phi = warm[3 * n + t];
-      // rho^w = 1 - phi (or the caller's rho^w field), rho^p = phi rho_f / rho_p, as
-      // deviations from the initial values
-      drw = (warm_rho ? (double)warm[4 * n + t] : 1.0 - phi) - k.rho_w0_d;
-      drp = phi / k.fr_d - k.rho_p0_d;
-    } else {
-      th = 0.5 - ((double)i + 0.5) / (double)L.nx;
-    }
-    const double dth = th - (0.5 - ((double)i + 0.5) / (double)L.nx);
-    const double rw = k.rho_w0_d + drw, rp = k.rho_p0_d + drp;
-    const double usq = 1.5 * (ux * ux + uy * uy);
+__device__ __noinline__ void init_node_fp64(T* __restrict__ dst, const Layout& L,
+                                            const StepConsts& k, const float* __restrict__ warm,
+                                            int warm_rho, int i, int j) {
+  const size_t n = (size_t)L.nx * L.ny, t = (size_t)j * L.nx + i;
+  const double ux = warm[t], uy = warm[n + t], th = warm[2 * n + t], phi = warm[3 * n + t];
+  // rho^w = 1 - phi (or the caller's rho^w field), rho^p = phi rho_f / rho_p, as deviations from
+  // the initial values
+  const double drw = (warm_rho ? (double)warm[4 * n + t] : 1.0 - phi) - k.rho_w0_d;
+  const double drp = phi / k.fr_d - k.rho_p0_d;
+  const double dth = th - (0.5 - ((double)i + 0.5) / (double)L.nx);
+  const double rw = k.rho_w0_d + drw, rp = k.rho_p0_d + drp;
+  const double usq = 1.5 * (ux * ux + uy * uy);
+  const size_t o = (size_t)j * L.pitch + i;
+#pragma unroll
+  for (int q = 0; q < kQ; ++q) {
+    const double eu = (double)ex(q) * ux + (double)ey(q) * uy;
+    const double P = eu * (3.0 + 4.5 * eu) - usq;
+    const double W = q == 0 ? 4.0 / 9.0 : (q <= 4 ? 1.0 / 9.0 : 1.0 / 36.0);
+    dst[(size_t)q * L.plane + o] = Elem<T>::put((float)(W * (drw + rw * P)));
+    dst[(size_t)(kQ + q) * L.plane + o] = Elem<T>::put((float)(W * (drp + rp * P)));
+    const T g = Elem<T>::put((float)(W * (dth + th * P)));
+    dst[(size_t)(2 * kQ + q) * L.plane + o] = g;
+    if (L.np == kPlanes2) dst[(size_t)(3 * kQ + q) * L.plane + o] = g;
+  }
+}
+
+// Unevaluated sums h + l of two FP32 numbers (Dekker; products by fma): about 2^-46 relative to
+// the largest term.
+struct Two {
+  float h, l;
+};
+__device__ __forceinline__ Two fast_two(float a, float b) {  // |a| >= |b|
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ Two two_of(double x) {
+  const float h = (float)x;
+  return {h, (float)(x - (double)h)};
+}
+__device__ __forceinline__ Two operator+(Two a, Two b) {
+  float e;
+  const float s = two_sum(a.h, b.h, e);
+  return fast_two(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ Two operator-(Two a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ Two operator*(Two a, Two b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return fast_two(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
+}
+__device__ __forceinline__ Two times(Two a, float b) {
+  const float p = __fmul_rn(a.h, b);
+  return fast_two(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
+}
+__device__ __forceinline__ Two product(float a, float b) {
+  const float p = __fmul_rn(a, b);
+  return {p, __fmaf_rn(a, b, -p)};
+}
+
+// a / b from inv = 1 / b rounded to nearest: the product corrected by its remainder, which rounds
+// like the division itself (Markstein, IBM J. Res. Dev. 34, 1990).
+__device__ __forceinline__ double quotient(double a, double b, double inv) {
+  const double q = a * inv;
+  return __fma_rn(__fma_rn(-q, b, a), inv, q);
+}
+
+// The equilibria of the caller's fields, W_q (d + r P_q) with d the deviation and r the absolute
+// value of rho^w, rho^p and theta. GB300 does 2 FP64 operations per clock and SM against 128 in
+// FP32, and the 27 polynomials in FP64 (about 160 operations per node) were all that the fill
+// waited for: 276 us on 1024 x 1024, where its 130 MB take 19 us. So only the cancelling
+// subtractions stay in FP64; the polynomials run in pairs of FP32 numbers, and a value whose
+// rounding to FP32 their error could decide (Ziv's test: adding and subtracting a bound of the
+// error does not round to the same number) sends its node to init_node_fp64. The stored values
+// are therefore those of the FP64 evaluation; about one node in 2000 takes the second way.
+// 1024 x 1024: 276 us before, 105 us now, still bound by the conversions and subtractions that
+// stay in FP64 (its pipe 81 % active).
+template <class T>
+__global__ void __launch_bounds__(256)
+    init_kernel(T* __restrict__ dst, const Layout L, const StepConsts k,
+                const float* __restrict__ warm, int warm_rho) {
+  const uint32_t n = (uint32_t)L.nx * (uint32_t)L.ny;
+  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+    const int j = (int)(t / (uint32_t)L.nx), i = (int)(t - (uint32_t)j * (uint32_t)L.nx);
     const size_t o = (size_t)j * L.pitch + i;
+    if (!warm) {  // at rest on the conduction profile every deviation is zero
+      for (int p = 0; p < L.np; ++p) dst[(size_t)p * L.plane + o] = Elem<T>::put(0.0f);
+      continue;
+    }
+    const float ux = warm[t], uy = warm[(size_t)n + t], thf = warm[2 * (size_t)n + t];
+    const float phi = warm[3 * (size_t)n + t];
+    const float rwf = warm_rho ? warm[4 * (size_t)n + t] : 0.0f;
+    const double phid = phi;
+    const double dw = (warm_rho ? (double)rwf : 1.0 - phid) - k.rho_w0_d;
+    const double dp = quotient(phid, k.fr_d, k.inv_fr_d) - k.rho_p0_d;
+    const double dt =
+        (double)thf - (0.5 - quotient((double)i + 0.5, (double)L.nx, k.inv_nx_d));
+    Two d[3] = {two_of(dw), two_of(dp), two_of(dt)};
+    Two r[3];
+    r[0].h = warm_rho ? rwf : two_sum(1.0f, -phi, r[0].l);
+    if (warm_rho) r[0].l = 0.0f;
+    r[1] = times({k.inv_fr_h, k.inv_fr_l}, phi);
+    r[2] = {thf, 0.0f};
+    // P_q = 3 e.u + 4.5 (e.u)^2 - 1.5 u.u: the even part of each axis and diagonal, the odd part
+    const Two A = product(ux, ux), B = product(uy, uy), C = times(product(ux, uy), 9.0f);
+    const Two AB3 = times(A + B, 3.0f);
+    const Two even[5] = {times(A + B, -1.5f), times(A, 3.0f) + times(B, -1.5f),
+                         times(B, 3.0f) + times(A, -1.5f), AB3 + C, AB3 + -C};
+    float el, fl;
+    const float e1 = two_sum(ux, uy, el), e2 = two_sum(uy, -ux, fl);
+    const Two odd[5] = {{0.0f, 0.0f}, product(3.0f, ux), product(3.0f, uy),
+                        times({e1, el}, 3.0f), times({e2, fl}, 3.0f)};
+    // The terms of set s weigh at most |d| + |r| (odd and even parts of P); the pairs above err by
+    // at most about 2^-43 of that. Terms so small that FP32 underflow could spoil the low parts
+    // are in doubt from the start (all zero is exact); so is NaN, which fails every comparison.
+    const float pm = 3.0f * (fabsf(ux) + fabsf(uy)) + 7.5f * (A.h + B.h);
+    bool doubt = false;
+    float err[3];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+      const float weight = fabsf(d[s].h) + fabsf(r[s].h) * pm;
+      err[s] = 0x1p-42f * weight;
+      doubt = doubt || !(weight >= 0x1p-80f || weight == 0.0f);
+    }
 #pragma unroll
     for (int q = 0; q < kQ; ++q) {
-      const double eu = (double)ex(q) * ux + (double)ey(q) * uy;
-      const double P = eu * (3.0 + 4.5 * eu) - usq;
-      const double W = q == 0 ? 4.0 / 9.0 : (q <= 4 ? 1.0 / 9.0 : 1.0 / 36.0);
-      dst[(size_t)q * L.plane + o] = Elem<T>::put((float)(W * (drw + rw * P)));
-      dst[(size_t)(kQ + q) * L.plane + o] = Elem<T>::put((float)(W * (drp + rp * P)));
-      dst[(size_t)(2 * kQ + q) * L.plane + o] = Elem<T>::put((float)(W * (dth + th * P)));
-      if (L.np == kPlanes2)
-        dst[(size_t)(3 * kQ + q) * L.plane + o] = Elem<T>::put((float)(W * (dth + th * P)));
+      // q of (q, -q): 0, 1, 2, 5, 6 (e_6 = (-1, 1)); the odd part of -q is negated
+      const int pr = q == 0 ? 0 : (q == 1 || q == 3 ? 1 : (q == 2 || q == 4 ? 2 :
+                                                            (q == 5 || q == 7 ? 3 : 4)));
+      const bool minus = q == 3 || q == 4 || q == 7 || q == 8;
+      const Two P = q == 0 ? even[0] : even[pr] + (minus ? -odd[pr] : odd[pr]);
+      const double Wd = q == 0 ? 4.0 / 9.0 : (q <= 4 ? 1.0 / 9.0 : 1.0 / 36.0);
+      const Two W = {(float)Wd, (float)(Wd - (double)(float)Wd)};
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        const Two v = W * (d[s] + r[s] * P);
+        const float e = W.h * err[s];
+        doubt = doubt || !(__fadd_rn(v.h, __fadd_rn(v.l, e)) == v.h &&
+                           __fadd_rn(v.h, __fsub_rn(v.l, e)) == v.h);
+        const T out = Elem<T>::put(v.h);
+        dst[(size_t)(s * kQ + q) * L.plane + o] = out;
+        if (s == 2 && L.np == kPlanes2) dst[(size_t)(3 * kQ + q) * L.plane + o] = out;
+      }
     }
+    if (doubt) init_node_fp64<T>(dst, L, k, warm, warm_rho, i, j);
   }
 }
 
@@ -173,13 +289,6 @@ __global__ void __launch_bounds__(kWallThreads)
   acc[0] = wall[0];
   acc[1] = wall[1];
   block_reduce_store<kRedWidth>(acc, out + (size_t)blockIdx.x * kRedWidth);
-}
-
-// a + b = s + e exactly (Knuth's two-sum; no operation below can be contracted)
-__device__ __forceinline__ float two_sum(float a, float b, float& e) {
-  const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
-  return s;
 }
 
 // Adds nine stored populations of a node to an FP64 sum. GB300 does 2 FP64 operations per clock

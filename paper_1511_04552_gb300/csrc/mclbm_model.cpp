@@ -171,6 +171,10 @@ StepConsts fold_step_consts(int nx, int ny, double phi, double d_p, const mclbm_
   k.rho_w0_d = c.rho_w0;
   k.rho_p0_d = c.rho_p0;
   k.fr_d = fr;
+  k.inv_fr_d = 1.0 / fr;
+  k.inv_nx_d = 1.0 / nx;
+  k.inv_fr_h = (float)k.inv_fr_d;
+  k.inv_fr_l = (float)(k.inv_fr_d - (double)k.inv_fr_h);
   return k;
 }
 
