@@ -21,12 +21,12 @@
  *   and 1 - phi (the solver conserves both components' masses).
  * Parameters: one flat FP32 vector, per conv layer (e0..e4, d3..d0, out) W[Cout][Cin][3][3]
  *   then b[Cout], then W1[hidden][3], b1[hidden], W2[F][hidden], b2[F], F = 2(C4+C3+C2+C1+C0).
- * Every convolution is an im2col GEMM on the tensor cores with BF16 operands (activations,
+ * Every convolution is an implicit GEMM on the tensor cores with BF16 operands (activations,
  * weights, and in the backward pass the pre-activation gradient, each rounded to nearest) and
  * FP32 accumulation: the forward pass, the weight gradient, and the input gradient (for the
- * stride-1 layers as the convolution of the pre-activation gradient with the flipped,
- * transposed kernel; for the stride-2 layers as a GEMM into the column gradient and its
- * fixed-order gather); everything else (FiLM, SiLU, the conditioning MLP, loss, reductions,
+ * stride-1 layers the convolution of the pre-activation gradient with the flipped, transposed
+ * kernel; for the stride-2 layers one product per tap, a pixel's taps added in a fixed order);
+ * everything else (FiLM, SiLU, the conditioning MLP, loss, reductions,
  * Adam) runs in FP32 CUDA-core kernels with fixed-order sums (FP64 across blocks).
  *
  * Conventions: return MCLBM_OK (0) or a negative MCLBM_E* code (mclbm.h); the caller owns all
@@ -60,7 +60,7 @@ void mclbm_net_config_default(mclbm_net_config* cfg);
 /* Number of FP32 parameters; 0 for an invalid configuration. */
 int64_t mclbm_net_param_count(const mclbm_net_config* cfg);
 /* Bytes of the device workspace mclbm_net_bind needs (parameters, Adam moments, activations,
- * im2col buffers, gradients); 0 for an invalid configuration. */
+ * gradients, partial sums); 0 for an invalid configuration. */
 size_t mclbm_net_workspace_bytes(const mclbm_net_config* cfg);
 
 /* A network handle for the configuration (copied). Host-only: no device memory until
@@ -111,7 +111,7 @@ int mclbm_net_loss_grad(mclbm_net_t* net, int batch, const float* cond_dev,
 int mclbm_net_train_step(mclbm_net_t* net, int batch, const float* cond_dev,
                          const float* target_dev, float lr, double* loss);
 
-/* The tensor-core GEMM every convolution uses, exposed for tests:
+/* A tensor-core GEMM (the network's convolutions have kernels of their own):
  *   D[z][m][n] = sum over k in split z of A(m, k) B(n, k),   0 <= m < M, 0 <= n < N,
  * A(m, k) = a[m*lda + k] (a_kmajor != 0) or a[k*lda + m]; B(n, k) likewise with b, ldb;
  * BF16 operands, FP32 result d[z*split_stride + m*ldd + n]; K is cut into `splits` ranges of

@@ -21,7 +21,7 @@ using namespace mcl::net;
 namespace {
 
 constexpr int kNumLayers = 10;
-constexpr int kLossBlocks = 1024;
+constexpr int kLossChunks = 64;  // most pixel chunks per sample of the loss
 constexpr int kStatBlocks = 256;
 static_assert(kFields * kStatBlocks * 2 >= kShiftPartials,
               "the warm start's mean shifts reuse the field statistics' scratch");
@@ -32,17 +32,21 @@ struct Layer {
   int src1, src2;  // producing layer of each input source (-1: the geometry input X)
   int up;          // src1 is upsampled by 2
   // shapes
-  int H, W, Ho, Wo, kin, Kp, splits;
-  int fsplits;  // forward split over K (layers with few output tiles), 1 otherwise
-  // input gradient as a convolution of the output gradient (stride 1, 9 cout <= Kp): the
-  // flipped, transposed kernel wt [cin][kp2], kp2 = 9 cout rounded up to 8
-  int tconv, kp2;
+  int H, W, Ho, Wo, kin;
+  int groups;      // channel groups of 8 of the input
+  int og;          // channel groups of the output
+  int fsplits, fsplit_k;  // forward split over K (layers with few output tiles): count, k each
   int64_t w_off, b_off;
   int film_off;  // offset of this layer's (gamma, beta) slice in r, or -1
+  // the layer that reads y, the channel group it is written at there, upsampled or not
+  int dst, dst_group, dst_up;
+  size_t wf_elems, wd_elems;  // packed weights: forward, input gradient
+  size_t sums_elems;
   // device buffers
-  float *pre, *y, *dy;
-  __nv_bfloat16 *cols, *wb, *dpre, *wt;
-  double* partial;
+  float *pre, *dy;
+  __nv_bfloat16 *in, *wf, *wd, *dpre;  // in: null for the stride-2 layers (they read a skip source)
+  float* part;
+  double* sums;
 };
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -55,16 +59,22 @@ struct mclbm_net {
   int F = 0;
   int64_t n_params = 0, mlp_off = 0;
   size_t ws_bytes = 0;
-  size_t dcols_elems = 0, wpart_elems = 0;
+  size_t wpart_elems = 0;  // partial sums of the weight gradients
+  size_t fpart_elems = 0;  // partial sums of the K-split forward layers
+  int sms = 152;           // multiprocessors, set by bind
   // bound memory
   char* ws = nullptr;
   cudaStream_t stream = nullptr;
   float *params = nullptr, *grads = nullptr, *adam_m = nullptr, *adam_v = nullptr;
   float* norm = nullptr;  // mean[5], scale[5] of the fields' deviations from their rest values
-  float* X = nullptr;
-  float *dcols = nullptr, *wpart = nullptr;
+  float *wpart = nullptr, *fpart = nullptr;
   float *cond_c = nullptr, *a1 = nullptr, *r = nullptr, *dr = nullptr;
   double *loss_part = nullptr, *loss = nullptr, *stat_part = nullptr;
+  // tensor maps and plans of the backward pass, laid out for one batch size
+  int plan_batch = 0;
+  WgradMaps wg_maps[kNumLayers];
+  WgradArgs wg[kNumLayers];
+  CUtensorMap dx_map[kNumLayers];
   int* err = nullptr;
   int adam_t = 0;
   bool bound = false;
@@ -93,6 +103,18 @@ bool config_valid(const mclbm_net_config* c) {
          c->hidden <= 256 && c->max_batch >= 1 && c->max_batch <= 256 &&
          (int64_t)c->max_batch * c->ny * c->nx <= (int64_t)1 << 26 &&
          c->max_batch * c->hidden <= 4096;  // the MLP kernels keep [batch][hidden] in shared memory
+}
+
+// Elements of a packed weight operand with n columns and K groups of 8 channels (see PackSeg).
+size_t packed_elems(int n, int groups) {
+  const int nt = conv_n_tile(n);
+  return (size_t)((n + nt - 1) / nt) * conv_slices(groups) * 18 * nt * 8;
+}
+
+// Elements of the layer's own input buffer: one image of the geometry, or the sources of a batch.
+size_t in_elems(const mclbm_net* n, int l) {
+  const Layer& y = n->L[l];
+  return (size_t)y.groups * 8 * y.H * y.W * (l == 0 ? 1 : n->cfg.max_batch);
 }
 
 // Layer table, parameter offsets and workspace size (no device work).
@@ -137,9 +159,9 @@ void plan(mclbm_net* n) {
     y.Ho = y.H / y.stride;
     y.Wo = y.W / y.stride;
     y.kin = 9 * (y.cu + y.cs);
-    y.Kp = (y.kin + 7) & ~7;
-    y.kp2 = (9 * y.cout + 7) & ~7;
-    y.tconv = l > 0 && y.stride == 1 && y.kp2 <= y.Kp;
+    y.groups = (y.cu + y.cs + 7) / 8;
+    y.og = (y.cout + 7) / 8;
+    y.dst = -1;
     y.w_off = off;
     off += (int64_t)y.cout * y.kin;
     y.b_off = off;
@@ -149,18 +171,30 @@ void plan(mclbm_net* n) {
       y.film_off = film_off;
       film_off += 2 * y.cout;
     }
-    const int tiles = ((y.cout + 127) / 128) * ((y.Kp + 127) / 128);
-    // weight gradient split over pixels so that its tiles fill one wave of the persistent GEMM
-    // (one CTA per SM with an MN-major B; 152 SMs on GB300); it changes only the order in which
-    // the FP32 partial sums are added
-    y.splits = std::max(1, std::min(64, 152 / tiles));
-    // forward GEMMs with fewer output tiles than half a wave are split over K as well (partial
-    // sums reduced in a fixed order by the epilogue kernel)
+    // forward products with fewer output tiles than half a wave (128 pixels x 128 channels each)
+    // are split over K in multiples of 64, partial sums added in order by the epilogue kernel
     const int64_t tiles_f = (((int64_t)c.max_batch * y.Ho * y.Wo + 127) / 128) *
                             ((y.cout + 127) / 128);
-    const int nks = (y.Kp + 63) / 64;
+    const int nks = (((y.kin + 7) & ~7) + 63) / 64;
     y.fsplits = tiles_f >= 76 ? 1 : (int)std::max<int64_t>(
                                         1, std::min<int64_t>({152 / tiles_f, 8, (int64_t)nks}));
+    y.fsplit_k = (nks + y.fsplits - 1) / y.fsplits * 64;
+  }
+  // where each layer's output goes: a decoder input (upsampled source first, then the skip
+  // source) or the output layer's; the stride-2 layers read the skip source where it lies
+  for (int l = 0; l < kNumLayers; ++l) {
+    const Layer& y = n->L[l];
+    if (y.stride == 2) continue;
+    if (y.src1 >= 0) {
+      n->L[y.src1].dst = l;
+      n->L[y.src1].dst_group = 0;
+      n->L[y.src1].dst_up = y.up;
+    }
+    if (y.src2 >= 0) {
+      n->L[y.src2].dst = l;
+      n->L[y.src2].dst_group = y.cu / 8;
+      n->L[y.src2].dst_up = 0;
+    }
   }
   n->F = film_off;
   n->mlp_off = off;
@@ -173,28 +207,37 @@ void plan(mclbm_net* n) {
   const size_t np = (size_t)n->n_params;
   bytes += 4 * align256(np * 4);  // params, grads, adam m, v
   bytes += align256(2 * kFields * 4);  // normaliser
-  bytes += align256((size_t)4 * B * c.ny * c.nx * 4);  // X
-  n->dcols_elems = 0;
   n->wpart_elems = 0;
+  n->fpart_elems = 0;
   for (int l = 0; l < kNumLayers; ++l) {
-    const Layer& y = n->L[l];
+    Layer& y = n->L[l];
     const size_t P = (size_t)B * y.Ho * y.Wo;
-    bytes += 3 * align256((size_t)y.cout * P * 4);           // pre, y, dy
-    bytes += align256(P * y.Kp * 2);                         // cols
-    bytes += align256((size_t)y.cout * y.Kp * 2);            // wb
-    if (y.tconv) bytes += align256((size_t)(y.cu + y.cs) * y.kp2 * 2);  // wt
-    bytes += align256((size_t)y.cout * P * 2);               // dpre
-    bytes += align256((size_t)y.cout * B * 3 * 8);           // partial
-    if (l > 0) n->dcols_elems = std::max(n->dcols_elems, P * y.Kp);
-    n->wpart_elems = std::max(n->wpart_elems, (size_t)y.splits * y.cout * y.Kp);
+    const int cin = y.cu + y.cs;
+    y.wf_elems = packed_elems(y.cout, y.groups);
+    y.wd_elems = l == 0 ? 0
+                 : y.stride == 1
+                     ? packed_elems(cin, y.og)
+                     : (size_t)((cin + 15) / 16) * ((y.og + dx_stride2_kg(y.cout) - 1) /
+                                                    dx_stride2_kg(y.cout)) *
+                           9 * dx_stride2_kg(y.cout) * 16 * 8;
+    // act_chunks is at most 608 / groups per batch, or 1 per sample
+    y.sums_elems = (size_t)y.cout * (std::max<size_t>(B, 608) + B * kLossChunks * (l == 9)) * 3;
+    bytes += align256((size_t)y.cout * P * 4);               // pre
+    bytes += align256((size_t)y.cout * P * 4);               // dy
+    if (y.stride == 1) bytes += align256(in_elems(n, l) * 2);  // in
+    bytes += align256(y.wf_elems * 2) + align256(y.wd_elems * 2);
+    bytes += align256((size_t)y.og * 8 * P * 2);             // dpre
+    bytes += align256(y.sums_elems * 8);
+    n->wpart_elems += wgrad_part_bound(y.groups, y.cout, y.kin, y.stride);
     if (y.fsplits > 1)
-      n->wpart_elems = std::max(n->wpart_elems, (size_t)y.fsplits * y.cout * P);
+      n->fpart_elems = std::max(n->fpart_elems, (size_t)y.fsplits * y.cout * P);
   }
-  bytes += align256(n->dcols_elems * 4);
   bytes += align256(n->wpart_elems * 4);
+  bytes += align256(n->fpart_elems * 4);
   bytes += align256((size_t)B * 3 * 4) + align256((size_t)B * c.hidden * 4) +
            2 * align256((size_t)B * n->F * 4);
-  bytes += align256(kLossBlocks * 8) + align256(8) + align256(kFields * kStatBlocks * 2 * 8);
+  bytes += align256((size_t)B * kLossChunks * 8) + align256(8) +
+           align256(kFields * kStatBlocks * 2 * 8);
   bytes += align256(4);
   n->ws_bytes = bytes;
 }
@@ -216,29 +259,33 @@ void assign(mclbm_net* n) {
   n->adam_m = carve<float>(p, np);
   n->adam_v = carve<float>(p, np);
   n->norm = carve<float>(p, 2 * kFields);
-  n->X = carve<float>(p, (size_t)4 * B * c.ny * c.nx);
   for (int l = 0; l < kNumLayers; ++l) {
     Layer& y = n->L[l];
     const size_t P = (size_t)B * y.Ho * y.Wo;
     y.pre = carve<float>(p, (size_t)y.cout * P);
-    y.y = carve<float>(p, (size_t)y.cout * P);
     y.dy = carve<float>(p, (size_t)y.cout * P);
-    y.cols = carve<__nv_bfloat16>(p, P * y.Kp);
-    y.wb = carve<__nv_bfloat16>(p, (size_t)y.cout * y.Kp);
-    y.wt = y.tconv ? carve<__nv_bfloat16>(p, (size_t)(y.cu + y.cs) * y.kp2) : nullptr;
-    y.dpre = carve<__nv_bfloat16>(p, (size_t)y.cout * P);
-    y.partial = carve<double>(p, (size_t)y.cout * B * 3);
+    y.in = y.stride == 1 ? carve<__nv_bfloat16>(p, in_elems(n, l)) : nullptr;
+    y.wf = carve<__nv_bfloat16>(p, y.wf_elems);
+    y.wd = carve<__nv_bfloat16>(p, y.wd_elems);
+    y.dpre = carve<__nv_bfloat16>(p, (size_t)y.og * 8 * P);
+    y.sums = carve<double>(p, y.sums_elems);
   }
-  n->dcols = carve<float>(p, n->dcols_elems);
   n->wpart = carve<float>(p, n->wpart_elems);
+  n->fpart = carve<float>(p, n->fpart_elems);
   n->cond_c = carve<float>(p, (size_t)B * 3);
   n->a1 = carve<float>(p, (size_t)B * c.hidden);
   n->r = carve<float>(p, (size_t)B * n->F);
   n->dr = carve<float>(p, (size_t)B * n->F);
-  n->loss_part = carve<double>(p, kLossBlocks);
+  n->loss_part = carve<double>(p, (size_t)B * kLossChunks);
   n->loss = carve<double>(p, 1);
   n->stat_part = carve<double>(p, kFields * kStatBlocks * 2);
   n->err = carve<int>(p, 1);
+  float* part = n->wpart;
+  for (int l = 0; l < kNumLayers; ++l) {
+    n->L[l].part = part;
+    part += wgrad_part_bound(n->L[l].groups, n->L[l].cout, n->L[l].kin, n->L[l].stride);
+  }
+  n->plan_batch = 0;
 }
 
 MlpArgs mlp_args(mclbm_net* n, int batch, const float* cond) {
@@ -259,92 +306,135 @@ MlpArgs mlp_args(mclbm_net* n, int batch, const float* cond) {
   return a;
 }
 
-const float* src_tensor(mclbm_net* n, int s) { return s < 0 ? n->X : n->L[s].y; }
-
+// BF16 weights in the operand layouts, from the FP32 parameters.
 cudaError_t refresh_bf16_weights(mclbm_net* n) {
+  PackArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.params = n->params;
   for (int l = 0; l < kNumLayers; ++l) {
     const Layer& y = n->L[l];
-    cudaError_t e = launch_weights_bf16(n->params + y.w_off, y.cout, y.kin, y.Kp, y.wb, n->stream);
+    for (int d = 0; d < (l == 0 ? 1 : 2); ++d) {
+      PackSeg& g = a.seg[a.count++];
+      g.kind = d == 0 ? kPackForward : (y.stride == 1 ? kPackTransposed : kPackStride2);
+      g.cout = y.cout;
+      g.cin = y.cu + y.cs;
+      g.nt = conv_n_tile(d == 0 ? y.cout : g.cin);
+      g.kg = dx_stride2_kg(y.cout);
+      g.slices = g.kind == kPackStride2 ? (y.og + g.kg - 1) / g.kg
+                                        : conv_slices(d == 0 ? y.groups : y.og);
+      g.w_off = y.w_off;
+      g.start = a.total;
+      g.out = d == 0 ? y.wf : y.wd;
+      a.total += (int64_t)(d == 0 ? y.wf_elems : y.wd_elems);
+    }
+  }
+  return launch_pack_weights(a, n->stream);
+}
+
+// A layer's input: its own buffer, or the skip source inside a decoder's input.
+struct Input {
+  const __nv_bfloat16* x;
+  int64_t group, image;  // pixels between groups and images
+};
+Input input_of(const mclbm_net* n, int l, int batch) {
+  const Layer& y = n->L[l];
+  const int64_t hw = (int64_t)y.H * y.W;
+  if (l == 0) return {y.in, hw, 0};
+  if (y.stride == 1) return {y.in, batch * hw, hw};
+  const Layer& s = n->L[y.src1];
+  return {n->L[s.dst].in + s.dst_group * batch * hw * 8, batch * hw, hw};
+}
+
+cudaError_t forward(mclbm_net* n, int batch, const float* cond, bool keep_pre) {
+  cudaStream_t st = n->stream;
+  cudaError_t e = launch_mlp_forward(mlp_args(n, batch, cond), st);
+  if (e != cudaSuccess) return e;
+  for (int l = 0; l < kNumLayers; ++l) {
+    Layer& y = n->L[l];
+    const Input in = input_of(n, l, batch);
+    ConvArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.src = in.x;
+    a.src_group = in.group;
+    a.src_image = in.image;
+    a.groups = y.groups;
+    a.batch = batch;
+    a.H = y.H;
+    a.W = y.W;
+    a.stride = y.stride;
+    a.Ho = y.Ho;
+    a.Wo = y.Wo;
+    a.N = y.cout;
+    a.w = y.wf;
+    a.err = n->err;
+    ConvEpilogue& ep = a.ep;
+    ep.bias = n->params + y.b_off;
+    ep.film = y.film ? n->r : nullptr;
+    ep.film_stride = n->F;
+    ep.film_off = y.film_off;
+    // the pre-activations are what the backward pass reads (and the output layer's the result)
+    ep.pre = keep_pre || l == kNumLayers - 1 ? y.pre : nullptr;
+    ep.act = y.act;
+    if (y.dst >= 0) {
+      const Layer& d = n->L[y.dst];
+      ep.y_group = (int64_t)batch * d.H * d.W;
+      ep.y = d.in + y.dst_group * ep.y_group * 8;
+      ep.up = y.dst_up;
+    }
+    plan_conv(&a, y.fsplits, y.fsplit_k);
+    if (y.fsplits > 1) {
+      a.part = n->fpart;
+      if ((e = launch_conv(a, kConvPartial, n->sms, st)) != cudaSuccess) return e;
+      e = launch_conv_epilogue_splitk(n->fpart, y.fsplits, batch, y.Ho, y.Wo, y.cout, ep, st);
+    } else {
+      e = launch_conv(a, kConvForward, n->sms, st);
+    }
     if (e != cudaSuccess) return e;
-    if (y.tconv &&
-        (e = launch_weights_t_bf16(n->params + y.w_off, y.cout, y.cu + y.cs, y.kp2, y.wt,
-                                   n->stream)) != cudaSuccess)
-      return e;
   }
   return cudaSuccess;
 }
 
-cudaError_t forward(mclbm_net* n, int batch, const float* cond) {
-  cudaStream_t st = n->stream;
-  cudaError_t e = launch_geometry(n->X, batch, n->cfg.ny, n->cfg.nx, st);
-  if (e != cudaSuccess) return e;
-  e = launch_mlp_forward(mlp_args(n, batch, cond), st);
-  if (e != cudaSuccess) return e;
+// Tensor maps and plans of the backward pass for a batch size (kept until another is asked for).
+bool plan_backward(mclbm_net* n, int batch) {
+  if (n->plan_batch == batch) return true;
+  n->plan_batch = 0;
   for (int l = 0; l < kNumLayers; ++l) {
-    Layer& y = n->L[l];
-    Im2colArgs ia;
-    ia.src1 = src_tensor(n, y.src1);
-    ia.src2 = y.src2 >= 0 ? n->L[y.src2].y : nullptr;
-    ia.cu = y.cu;
-    ia.cs = y.cs;
-    ia.up = y.up;
-    ia.batch = batch;
-    ia.H = y.H;
-    ia.W = y.W;
-    ia.stride = y.stride;
-    ia.Ho = y.Ho;
-    ia.Wo = y.Wo;
-    ia.Kp = y.Kp;
-    ia.cols = y.cols;
-    if ((e = launch_im2col(ia, st)) != cudaSuccess) return e;
-    const int P = batch * y.Ho * y.Wo;
-    GemmArgs g;
-    std::memset(&g, 0, sizeof(g));
-    g.a = y.cols;
-    g.lda = y.Kp;
-    g.a_kmajor = 1;
-    g.b = y.wb;
-    g.ldb = y.Kp;
-    g.b_kmajor = 1;
-    g.M = P;
-    g.N = y.cout;
-    g.K = y.Kp;
-    g.ep.bias = n->params + y.b_off;
-    g.ep.film = y.film ? n->r : nullptr;
-    g.ep.film_stride = n->F;
-    g.ep.film_off = y.film_off;
-    g.ep.hw = y.Ho * y.Wo;
-    g.ep.pre = y.pre;
-    g.ep.y = l == kNumLayers - 1 ? nullptr : y.y;
-    g.ep.act = y.act;
-    g.err = n->err;
-    if (y.fsplits > 1) {
-      // partial products per K split, column-major [split][cout][P], then the epilogue
-      const int nks = (y.Kp + 63) / 64;
-      g.k_per_split = (int64_t)((nks + y.fsplits - 1) / y.fsplits) * 64;
-      g.mode = kGemmRaw;
-      g.d = n->wpart;
-      g.ldd = P;
-      g.d_trans = 1;
-      g.split_stride = (int64_t)y.cout * P;
-      if ((e = launch_gemm(g, y.fsplits, st)) != cudaSuccess) return e;
-      if ((e = launch_conv_epilogue_splitk(n->wpart, y.fsplits, g.split_stride, P, y.cout, g.ep,
-                                           st)) != cudaSuccess)
-        return e;
+    const Layer& y = n->L[l];
+    const int64_t P = (int64_t)batch * y.Ho * y.Wo;
+    WgradArgs& a = n->wg[l];
+    std::memset(&a, 0, sizeof(a));
+    plan_wgrad(&a, y.groups, y.cout, y.kin, y.Ho, y.Wo, batch, y.stride, n->sms);
+    a.src_images = l > 0;
+    a.part = y.part;
+    a.err = n->err;
+    WgradMaps& m = n->wg_maps[l];
+    if (!encode_groups(&m.a, y.dpre, y.og, P, batch, y.Ho, y.Wo, 8, a.go, 16)) return false;
+    const Input in = input_of(n, l, batch);
+    const int images = l == 0 ? 1 : batch;
+    if (y.stride == 1) {
+      if (!encode_groups(&m.b[0], in.x, y.groups, in.group, images, y.H, y.W, 10, a.gc, 18))
+        return false;
     } else {
-      g.k_per_split = ((y.Kp + 63) / 64) * 64;
-      g.mode = kGemmConvFwd;
-      if ((e = launch_gemm(g, 1, st)) != cudaSuccess) return e;
+      for (int p = 0; p < 4; ++p)
+        if (!encode_parity(&m.b[p], in.x, p >> 1, p & 1, y.groups, in.group, images, y.H, y.W, 9,
+                           a.gc, 17))
+          return false;
+      if (!encode_groups(&n->dx_map[l], y.dpre, y.og, P, batch, y.Ho, y.Wo, 9,
+                         dx_stride2_kg(y.cout), 17))
+        return false;
     }
   }
-  return cudaSuccess;
+  n->plan_batch = batch;
+  return true;
 }
 
 // Loss and gradients into n->grads (loss into n->loss on the device).
 cudaError_t loss_backward(mclbm_net* n, int batch, const float* cond, const float* target) {
   cudaStream_t st = n->stream;
+  if (!plan_backward(n, batch)) return cudaErrorNotSupported;
   const int hw = n->cfg.ny * n->cfg.nx;
   Layer& out = n->L[kNumLayers - 1];
+  int sum_chunks[kNumLayers];
   LossArgs la;
   la.out = out.pre;
   la.target = target;
@@ -352,147 +442,112 @@ cudaError_t loss_backward(mclbm_net* n, int batch, const float* cond, const floa
   la.norm = n->norm;
   la.batch = batch;
   la.hw = hw;
-  la.dout = out.dy;
+  la.chunks = std::min(kLossChunks, act_chunks(8, batch, hw));
+  la.dpre = out.dpre;
+  la.sums = out.sums;
   la.partial = n->loss_part;
-  la.blocks = kLossBlocks;
+  sum_chunks[kNumLayers - 1] = la.chunks;
   cudaError_t e = launch_loss(la, st);
   if (e != cudaSuccess) return e;
-  if ((e = launch_sum_partials(n->loss_part, kLossBlocks, n->loss, st)) != cudaSuccess) return e;
+  if ((e = launch_sum_partials(n->loss_part, batch * la.chunks, n->loss, st)) != cudaSuccess)
+    return e;
 
   bool written[kNumLayers] = {false};
   for (int l = kNumLayers - 1; l >= 0; --l) {
     Layer& y = n->L[l];
-    const int P = batch * y.Ho * y.Wo;
-    ActBwdArgs aa;
-    aa.dy = y.dy;
-    aa.pre = y.pre;
-    aa.film = y.film ? n->r : nullptr;
-    aa.film_stride = n->F;
-    aa.film_off = y.film_off;
-    aa.C = y.cout;
-    aa.batch = batch;
-    aa.hw = y.Ho * y.Wo;
-    aa.act = y.act;
-    aa.dpre = y.dpre;
-    aa.partial = y.partial;
-    if ((e = launch_act_backward(aa, st)) != cudaSuccess) return e;
-    if ((e = launch_bias_film_grad(y.partial, y.cout, batch, n->grads + y.b_off,
-                                   y.film ? n->dr : nullptr, n->F, y.film_off, st)) != cudaSuccess)
-      return e;
-    // weight gradient: dW[o][k] = sum_p dpre[o][p] cols[p][k], split over p
-    GemmArgs g;
-    std::memset(&g, 0, sizeof(g));
-    g.a = y.dpre;
-    g.lda = P;
-    g.a_kmajor = 1;
-    g.b = y.cols;
-    g.ldb = y.Kp;
-    g.b_kmajor = 0;
-    g.M = y.cout;
-    g.N = y.Kp;
-    g.K = P;
-    g.k_per_split = ((((int64_t)P + y.splits - 1) / y.splits + 63) / 64) * 64;
-    g.d = n->wpart;
-    g.ldd = y.Kp;
-    g.split_stride = (int64_t)y.cout * y.Kp;
-    g.mode = kGemmRaw;
-    g.err = n->err;
-    if ((e = launch_gemm(g, y.splits, st)) != cudaSuccess) return e;
-    if ((e = launch_splitk_reduce(n->wpart, y.splits, g.split_stride, y.cout, y.kin, y.Kp,
-                                  n->grads + y.w_off, st)) != cudaSuccess)
-      return e;
+    if (l < kNumLayers - 1) {
+      ActBwdArgs aa;
+      aa.dy = y.dy;
+      aa.pre = y.pre;
+      aa.film = y.film ? n->r : nullptr;
+      aa.film_stride = n->F;
+      aa.film_off = y.film_off;
+      aa.C = y.cout;
+      aa.batch = batch;
+      aa.hw = y.Ho * y.Wo;
+      aa.chunks = act_chunks(y.cout, batch, aa.hw);
+      aa.dpre = y.dpre;
+      aa.sums = y.sums;
+      sum_chunks[l] = aa.chunks;
+      if ((e = launch_act_backward(aa, st)) != cudaSuccess) return e;
+    }
+    if ((e = launch_wgrad(n->wg_maps[l], n->wg[l], st)) != cudaSuccess) return e;
     if (l == 0) break;
-    if (y.tconv) {
-      // input gradient of a stride-1 convolution as the convolution of the output gradient with
-      // the flipped, transposed kernel: dX[c][q] = sum_(o, t) wt[c][o 9 + t] cols2[q][o 9 + t],
-      // cols2 the im2col rows of dpre (in this layer's cols buffer), then routed to the sources
-      Im2colBf16Args ib;
-      ib.src = y.dpre;
-      ib.C = y.cout;
-      ib.batch = batch;
-      ib.H = y.Ho;
-      ib.W = y.Wo;
-      ib.Kp = y.kp2;
-      ib.cols = y.cols;
-      if ((e = launch_im2col_bf16(ib, st)) != cudaSuccess) return e;
-      std::memset(&g, 0, sizeof(g));
-      g.a = y.cols;
-      g.lda = y.kp2;
-      g.a_kmajor = 1;
-      g.b = y.wt;
-      g.ldb = y.kp2;
-      g.b_kmajor = 1;
-      g.M = P;
-      g.N = y.cu + y.cs;
-      g.K = y.kp2;
-      g.k_per_split = ((y.kp2 + 63) / 64) * 64;
-      g.d = n->dcols;
-      g.ldd = P;
-      g.d_trans = 1;
-      g.mode = kGemmRaw;
-      g.err = n->err;
-      if ((e = launch_gemm(g, 1, st)) != cudaSuccess) return e;
-      RouteArgs ra;
-      ra.dx = n->dcols;
-      ra.cu = y.cu;
-      ra.cs = y.src2 >= 0 ? y.cs : 0;
-      ra.up = y.up;
-      ra.batch = batch;
-      ra.H = y.H;
-      ra.W = y.W;
-      ra.dsrc1 = n->L[y.src1].dy;
-      ra.acc1 = written[y.src1] ? 1 : 0;
+    if (y.stride == 2) {
+      DxStride2Args d;
+      std::memset(&d, 0, sizeof(d));
+      d.batch = batch;
+      d.Ho = y.Ho;
+      d.Wo = y.Wo;
+      d.C = y.cu;
+      d.w = y.wd;
+      d.dsrc = n->L[y.src1].dy;
+      d.accumulate = written[y.src1] ? 1 : 0;
       written[y.src1] = true;
-      ra.dsrc2 = nullptr;
-      ra.acc2 = 0;
-      if (y.src2 >= 0) {
-        ra.dsrc2 = n->L[y.src2].dy;
-        ra.acc2 = written[y.src2] ? 1 : 0;
-        written[y.src2] = true;
-      }
-      if ((e = launch_route_grad(ra, st)) != cudaSuccess) return e;
+      d.err = n->err;
+      plan_dx_stride2(&d, y.cout);
+      if ((e = launch_dx_stride2(n->dx_map[l], d, n->sms, st)) != cudaSuccess) return e;
       continue;
     }
-    // input gradient: dcols[k][p] = sum_o dpre[o][p] wb[o][k], stored column-major so that
-    // the epilogue's stores and col2im's reads are coalesced over pixels
-    std::memset(&g, 0, sizeof(g));
-    g.a = y.dpre;
-    g.lda = P;
-    g.a_kmajor = 0;
-    g.b = y.wb;
-    g.ldb = y.Kp;
-    g.b_kmajor = 0;
-    g.M = P;
-    g.N = y.Kp;
-    g.K = y.cout;
-    g.k_per_split = ((y.cout + 63) / 64) * 64;
-    g.d = n->dcols;
-    g.ldd = P;
-    g.d_trans = 1;
-    g.mode = kGemmRaw;
-    g.err = n->err;
-    if ((e = launch_gemm(g, 1, st)) != cudaSuccess) return e;
-    for (int s = 0; s < 2; ++s) {
-      const int src = s == 0 ? y.src1 : y.src2;
-      if (s == 1 && src < 0) break;
-      Col2imArgs ca;
-      ca.dcols = n->dcols;
-      ca.Kp = y.Kp;
-      ca.c_lo = s == 0 ? 0 : y.cu;
-      ca.C = s == 0 ? y.cu : y.cs;
-      ca.up = s == 0 ? y.up : 0;
-      ca.batch = batch;
-      ca.H = y.H;
-      ca.W = y.W;
-      ca.stride = y.stride;
-      ca.Ho = y.Ho;
-      ca.Wo = y.Wo;
-      ca.dsrc = n->L[src].dy;
-      ca.accumulate = written[src] ? 1 : 0;
-      written[src] = true;
-      if ((e = launch_col2im(ca, st)) != cudaSuccess) return e;
+    // the convolution of the pre-activation gradient with the flipped, transposed kernel
+    ConvArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.src = y.dpre;
+    a.src_image = (int64_t)y.Ho * y.Wo;
+    a.src_group = batch * a.src_image;
+    a.groups = y.og;
+    a.batch = batch;
+    a.H = a.Ho = y.Ho;
+    a.W = a.Wo = y.Wo;
+    a.stride = 1;
+    a.N = y.cu + y.cs;
+    a.w = y.wd;
+    a.err = n->err;
+    RouteArgs& ra = a.route;
+    ra.cu = y.cu;
+    ra.up = y.up;
+    ra.dsrc1 = n->L[y.src1].dy;
+    ra.acc1 = written[y.src1] ? 1 : 0;
+    written[y.src1] = true;
+    if (y.src2 >= 0) {
+      ra.dsrc2 = n->L[y.src2].dy;
+      ra.acc2 = written[y.src2] ? 1 : 0;
+      written[y.src2] = true;
     }
+    plan_conv(&a, 1, 0);
+    if ((e = launch_conv(a, kConvRoute, n->sms, st)) != cudaSuccess) return e;
   }
+
+  FinishArgs f;
+  std::memset(&f, 0, sizeof(f));
+  f.count = kNumLayers;
+  f.batch = batch;
+  f.film_stride = n->F;
+  f.dfilm = n->dr;
+  for (int l = 0; l < kNumLayers; ++l) {
+    const Layer& y = n->L[l];
+    const WgradArgs& a = n->wg[l];
+    FinishSeg& g = f.seg[l];
+    g.cout = y.cout;
+    g.kin = y.kin;
+    g.gc = a.gc;
+    g.s2 = a.s2;
+    g.chunks = a.chunks;
+    g.ochunks = a.ochunks;
+    g.cols = a.cols;
+    g.mrows = a.mrows;
+    g.splits = a.splits;
+    g.sum_chunks = sum_chunks[l];
+    g.film_off = y.film_off;
+    for (int k = 0; k < 6; ++k) g.col[k] = a.e[k].col;
+    g.start = f.total;
+    f.total += (int64_t)y.cout * y.kin;
+    g.part = y.part;
+    g.sums = y.sums;
+    g.grad = n->grads + y.w_off;
+    g.dbias = n->grads + y.b_off;
+  }
+  if ((e = launch_finish(f, st)) != cudaSuccess) return e;
   const MlpArgs ma = mlp_args(n, batch, nullptr);
   float* gW1 = n->grads + n->mlp_off;
   float* gb1 = gW1 + 3 * n->cfg.hidden;
@@ -591,6 +646,13 @@ int mclbm_net_bind(mclbm_net_t* n, void* ws, size_t bytes, void* stream) {
     norm[kFields + c] = 1.f;
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(n->norm, norm, sizeof(norm), cudaMemcpyHostToDevice, st);
+  // the geometry input stays as it is for the handle's life
+  int dev = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&n->sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = prepare_conv_kernels();
+  if (e == cudaSuccess) e = launch_geometry(n->L[0].in, n->cfg.ny, n->cfg.nx, st);
   if (e == cudaSuccess) e = refresh_bf16_weights(n);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(n, e, "mclbm_net_bind");
@@ -696,7 +758,7 @@ int mclbm_net_forward(mclbm_net_t* n, int batch, const float* cond, float* field
   int rc = check_call(n, batch);
   if (rc != MCLBM_OK) return rc;
   if (!cond || !fields) return fail(n, MCLBM_EINVAL, "null pointer");
-  cudaError_t e = forward(n, batch, cond);
+  cudaError_t e = forward(n, batch, cond, false);
   if (e == cudaSuccess)
     e = launch_denormalize(n->L[kNumLayers - 1].pre, n->norm, cond, batch,
                            n->cfg.ny * n->cfg.nx, n->stat_part, fields, n->stream);
@@ -709,7 +771,7 @@ int mclbm_net_loss_grad(mclbm_net_t* n, int batch, const float* cond, const floa
   int rc = check_call(n, batch);
   if (rc != MCLBM_OK) return rc;
   if (!cond || !target || !grad || !loss) return fail(n, MCLBM_EINVAL, "null pointer");
-  cudaError_t e = forward(n, batch, cond);
+  cudaError_t e = forward(n, batch, cond, true);
   if (e == cudaSuccess) e = loss_backward(n, batch, cond, target);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(grad, n->grads, (size_t)n->n_params * 4, cudaMemcpyDeviceToDevice,
@@ -724,7 +786,7 @@ int mclbm_net_train_step(mclbm_net_t* n, int batch, const float* cond, const flo
   int rc = check_call(n, batch);
   if (rc != MCLBM_OK) return rc;
   if (!cond || !target || !(lr > 0.f)) return fail(n, MCLBM_EINVAL, "bad argument");
-  cudaError_t e = forward(n, batch, cond);
+  cudaError_t e = forward(n, batch, cond, true);
   if (e == cudaSuccess) e = loss_backward(n, batch, cond, target);
   if (e == cudaSuccess) {
     n->adam_t += 1;
@@ -757,7 +819,6 @@ int mclbm_gemm_bf16(int M, int N, int K, const void* a, int64_t lda, int a_kmajo
   g.d = d;
   g.ldd = ldd;
   g.split_stride = split_stride;
-  g.mode = kGemmRaw;
   g.err = nullptr;
   if (!gemm_args_valid(g, splits)) return MCLBM_EINVAL;
   return launch_gemm(g, splits, static_cast<cudaStream_t>(stream)) == cudaSuccess ? MCLBM_OK

@@ -1,6 +1,4 @@
-// BF16 tensor-core GEMM on the 5th-generation tensor cores (tcgen05), the contraction behind
-// every convolution of the warm-start network: forward (im2col rows x weights), input gradient
-// (output gradient x weights) and weight gradient (output gradient x im2col, split over K).
+// BF16 tensor-core GEMM on the 5th-generation tensor cores (tcgen05), mclbm_gemm_bf16.
 //
 // A persistent grid (every resident CTA slot, at most one CTA per tile) of 128-thread CTAs walks
 // the 128 x 128 tiles of D = A B^T (and the K splits); for each tile:
@@ -17,8 +15,7 @@
 //    the FP32 accumulator in tensor memory (128 columns allocated per CTA) and commits them to
 //    the stage's mbarrier;
 //  * the four warps read the accumulator back with tcgen05.ld (warp w owns TMEM lanes
-//    32w..32w+31 = tile rows) and apply the epilogue (raw store or the convolution's bias,
-//    FiLM and SiLU, written channel-major so that consecutive threads write consecutive pixels).
+//    32w..32w+31 = tile rows) and store it.
 // Every mbarrier wait is bounded (2 s on %globaltimer); on timeout the CTA sets the error word,
 // waits (bounded) for its MMAs, frees its tensor memory and returns.
 #include <cuda.h>
@@ -30,6 +27,7 @@
 #include <cstdint>
 
 #include "net_internal.h"
+#include "net_tc.cuh"
 
 namespace mcl {
 namespace net {
@@ -49,97 +47,6 @@ __host__ __device__ constexpr int smem_bytes_for(int N) {
   return kStages * stage_stride_for(N) + 8 * kStages + 64;
 }
 constexpr uint32_t kTmemCols = 128;
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ uint64_t now_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ bool bar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Waits for the phase with the given parity; false after about 2 s.
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
-  if (bar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = now_ns();
-  for (uint32_t k = 0; k < (1u << 26); ++k) {
-    if (bar_try_wait(bar, parity)) return true;
-    if (now_ns() - t0 > 2000000000ull) return false;
-  }
-  return false;
-}
-
-// ---- tcgen05 wrappers ----------------------------------------------------------------------
-__device__ __forceinline__ void tmem_alloc(uint32_t slot_smem, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot_smem),
-               "r"(ncols)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
-               : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-// Shared-memory matrix descriptor: start address, leading (K-direction) and stride
-// (8-row-group) byte offsets, descriptor version 1, no swizzle.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
-// Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, A (bit 15) and B
-// (bit 16) K-major (0) or MN-major (1), N >> 3 at bit 17, M >> 4 at bit 24.
-__device__ __forceinline__ uint32_t instr_desc(int m, int n, bool a_mn, bool b_mn) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) |
-         ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-      : "memory");
-}
-// 16 consecutive FP32 accumulator columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-      "%11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
-}
 
 // Offset of element (r, k) of a staged 128 x 64 slice (canonical K-major, no swizzle).
 __device__ __forceinline__ uint32_t tile_off(int r, int k) {
@@ -299,41 +206,13 @@ __device__ __forceinline__ void store_operand(uint8_t* dst, const uint4 (&v)[kSt
 // persistent CTA takes tiles blockIdx.x, + gridDim.x, ... and the slices of all its tiles form
 // one stream through the stage ring, so the next tile's loads are in flight while a tile's
 // epilogue runs.
-// Epilogue of 16 accumulator columns n..n+15 of one row of D (split z): a raw store
-// (row-major, or column-major with d_trans: a warp's 32 rows are then 32 consecutive floats),
-// or the convolution's bias, FiLM and SiLU, written channel-major.
+// Epilogue of 16 accumulator columns n..n+15 of one row of D (split z).
 __device__ __forceinline__ void store_cols(const GemmArgs& g, int row, int n, int z,
                                            const float (&v)[16]) {
-  if (g.mode == kGemmRaw) {
-    float* d = g.d + (int64_t)z * g.split_stride;
-    if (g.d_trans) {
+  float* dst = g.d + (int64_t)z * g.split_stride + (int64_t)row * g.ldd + n;
 #pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (n + j < g.N) d[(int64_t)(n + j) * g.ldd + row] = v[j];
-    } else {
-      float* dst = d + (int64_t)row * g.ldd + n;
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (n + j < g.N) dst[j] = v[j];
-    }
-  } else {
-    const ConvEpilogue& e = g.ep;
-    const int b = row / e.hw;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int o = n + j;
-      if (o >= g.N) break;
-      const float pre = v[j] + e.bias[o];
-      float zz = pre;
-      if (e.film) {
-        const float* f = e.film + (int64_t)b * e.film_stride + e.film_off;
-        zz = (1.f + f[o]) * pre + f[g.N + o];
-      }
-      const int64_t idx = (int64_t)o * g.M + row;
-      e.pre[idx] = pre;
-      if (e.y) e.y[idx] = e.act ? zz / (1.f + expf(-zz)) : zz;
-    }
-  }
+  for (int j = 0; j < 16; ++j)
+    if (n + j < g.N) dst[j] = v[j];
 }
 
 struct TileCursor {
@@ -549,24 +428,6 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr, uint32_t lbo
          ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 
-__device__ __forceinline__ void bar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void bar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// a bounded wait that also gives up when another role has already given up
-__device__ __forceinline__ bool role_wait(uint32_t bar, uint32_t parity, volatile int* abort) {
-  if (bar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = now_ns();
-  for (uint32_t k = 0; k < (1u << 26); ++k) {
-    if (bar_try_wait(bar, parity)) return true;
-    if (*abort || now_ns() - t0 > 2000000000ull) return false;
-  }
-  return false;
-}
-
 __global__ void __launch_bounds__(kTmaThreads) gemm_bf16_tma_kernel(
     const __grid_constant__ TmaGemmMaps maps, const GemmArgs g) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -737,14 +598,8 @@ bool gemm_args_valid(const GemmArgs& g, int splits) {
   if ((int64_t)splits * g.k_per_split < g.K) return false;
   if (g.a_kmajor ? g.lda < g.K : g.lda < g.M) return false;
   if (g.b_kmajor ? g.ldb < g.K : g.ldb < g.N) return false;
-  if (g.mode == kGemmRaw) {
-    if (!g.d || g.ldd < (g.d_trans ? g.M : g.N)) return false;
-    if (splits > 1 && g.split_stride < (int64_t)(g.d_trans ? g.N : g.M) * g.ldd) return false;
-  } else if (g.mode == kGemmConvFwd) {
-    if (splits != 1 || !g.ep.bias || !g.ep.pre || g.ep.hw <= 0 || g.M % g.ep.hw) return false;
-  } else {
-    return false;
-  }
+  if (!g.d || g.ldd < g.N) return false;
+  if (splits > 1 && g.split_stride < (int64_t)g.M * g.ldd) return false;
   return true;
 }
 

@@ -1,10 +1,7 @@
-// CUDA-core kernels of the warm-start network around the tensor-core GEMM (net_gemm.cu):
-// im2col with fused nearest upsampling and channel concatenation, the input gradient of the
-// stride-1 layers as a convolution (im2col of the output gradient, the flipped kernel, routing
-// to the sources) and of the stride-2 layers by col2im as a gather (every input gradient summed
-// in a fixed order), the backward of FiLM + SiLU with
-// the per-channel reductions, the conditioning MLP, the loss, Adam, and small helpers.
-// Activations are channel-major: x[c][b * H * W + y * W + x].
+// CUDA-core kernels of the warm-start network around its convolutions (net_conv.cu): the backward
+// of FiLM + SiLU with the per-channel reductions, the epilogue of the K-split convolutions, the
+// conditioning MLP, the loss, Adam, the output's denormalisation and small helpers.
+// FP32 activations and gradients are channel-major, x[c][b * H * W + y * W + x].
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -13,6 +10,7 @@
 #include <cstdint>
 
 #include "net_internal.h"
+#include "net_tc.cuh"
 
 namespace mcl {
 namespace net {
@@ -51,330 +49,163 @@ __device__ __forceinline__ void block_sum(double* v, double (*sh)[NV]) {
   __syncthreads();
 }
 
-// ---- im2col ---------------------------------------------------------------------------------
-// One thread per (output pixel, group of 8 columns): 16-byte stores of BF16.
-__global__ void im2col_kernel(const Im2colArgs a) {
-  const int kg_n = a.Kp / 8;
-  const int64_t P = (int64_t)a.batch * a.Ho * a.Wo;
-  const int kin = 9 * (a.cu + a.cs);
-  const int H1 = a.up ? a.H / 2 : a.H, W1 = a.up ? a.W / 2 : a.W;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < P * kg_n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int kg = (int)(t % kg_n);
-    const int64_t p = t / kg_n;
-    const int xo = (int)(p % a.Wo);
-    const int yo = (int)((p / a.Wo) % a.Ho);
-    const int b = (int)(p / ((int64_t)a.Wo * a.Ho));
-    __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int k = kg * 8 + j;
-      float x = 0.f;
-      if (k < kin) {
-        const int c = k / 9, tap = k - 9 * c;
-        const int yi = a.stride * yo + tap / 3 - 1, xi = a.stride * xo + tap % 3 - 1;
-        if (yi >= 0 && yi < a.H && xi >= 0 && xi < a.W) {
-          if (c < a.cu) {
-            const int ys = a.up ? yi >> 1 : yi, xs = a.up ? xi >> 1 : xi;
-            x = a.src1[((int64_t)c * a.batch + b) * H1 * W1 + (int64_t)ys * W1 + xs];
-          } else {
-            x = a.src2[((int64_t)(c - a.cu) * a.batch + b) * a.H * a.W + (int64_t)yi * a.W + xi];
-          }
-        }
-      }
-      v[j] = __float2bfloat16_rn(x);
-    }
-    *reinterpret_cast<uint4*>(a.cols + p * a.Kp + kg * 8) = *reinterpret_cast<const uint4*>(v);
-  }
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  uint32_t u;
+  memcpy(&u, &v, 4);
+  return u;
 }
 
-// Channel counts in multiples of 8 (every layer but the geometry input): one thread per (output
-// pixel, group of 8 channels) writes the group's 72 columns (c 9 + tap, 144 contiguous bytes)
-// as nine 16-byte stores; consecutive threads take consecutive pixels of one group, so every
-// load of a warp reads consecutive pixels of one channel and tap.
-__global__ void im2col_c8_kernel(const Im2colArgs a) {
-  const int cg_n = (a.cu + a.cs) / 8;
-  const int64_t P = (int64_t)a.batch * a.Ho * a.Wo;
-  const int H1 = a.up ? a.H / 2 : a.H, W1 = a.up ? a.W / 2 : a.W;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < P * cg_n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = t % P;
-    const int cg = (int)(t / P);
-    const int xo = (int)(p % a.Wo);
-    const int yo = (int)((p / a.Wo) % a.Ho);
-    const int b = (int)(p / ((int64_t)a.Wo * a.Ho));
-    __align__(16) __nv_bfloat16 v[72];
+// A sum of FP32 terms with the exact errors of its additions beside it (Knuth's two-sum).
+struct Sum {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)));
+    s = t;
+  }
+};
+
+// The lane-0 sums of a warp's N compensated sums: FP32 pairs in a fixed order (FP64 runs at 1/64
+// of the FP32 rate).
+template <int N>
+__device__ __forceinline__ void warp_sums(Sum (&v)[N], double* out) {
 #pragma unroll
-    for (int cc = 0; cc < 8; ++cc) {
-      const int c = cg * 8 + cc;
-#pragma unroll
-      for (int tap = 0; tap < 9; ++tap) {
-        const int yi = a.stride * yo + tap / 3 - 1, xi = a.stride * xo + tap % 3 - 1;
-        float x = 0.f;
-        if (yi >= 0 && yi < a.H && xi >= 0 && xi < a.W) {
-          if (c < a.cu) {
-            const int ys = a.up ? yi >> 1 : yi, xs = a.up ? xi >> 1 : xi;
-            x = a.src1[((int64_t)c * a.batch + b) * H1 * W1 + (int64_t)ys * W1 + xs];
-          } else {
-            x = a.src2[((int64_t)(c - a.cu) * a.batch + b) * a.H * a.W + (int64_t)yi * a.W + xi];
-          }
-        }
-        v[cc * 9 + tap] = __float2bfloat16_rn(x);
-      }
+  for (int k = 0; k < N; ++k) {
+    for (int off = 16; off > 0; off >>= 1) {
+      const float s = __shfl_down_sync(0xffffffffu, v[k].s, off);
+      const float e = __shfl_down_sync(0xffffffffu, v[k].e, off);
+      v[k].add(s);
+      v[k].e = __fadd_rn(v[k].e, e);
     }
-    uint4* dst = reinterpret_cast<uint4*>(a.cols + p * a.Kp + cg * 72);
-#pragma unroll
-    for (int q = 0; q < 9; ++q) dst[q] = reinterpret_cast<const uint4*>(v)[q];
+    if ((threadIdx.x & 31) == 0) out[k] = (double)v[k].s + (double)v[k].e;
   }
 }
-
-// ---- input gradient as a convolution (stride-1 layers) --------------------------------------
-__global__ void im2col_bf16_kernel(const Im2colBf16Args a) {
-  const int kg_n = a.Kp / 8;
-  const int64_t P = (int64_t)a.batch * a.H * a.W;
-  const int kin = 9 * a.C;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < P * kg_n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int kg = (int)(t % kg_n);
-    const int64_t p = t / kg_n;
-    const int x = (int)(p % a.W);
-    const int y = (int)((p / a.W) % a.H);
-    const int b = (int)(p / ((int64_t)a.W * a.H));
-    __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int k = kg * 8 + j;
-      __nv_bfloat16 s = __float2bfloat16_rn(0.f);
-      if (k < kin) {
-        const int c = k / 9, tap = k - 9 * c;
-        const int yi = y + tap / 3 - 1, xi = x + tap % 3 - 1;
-        if (yi >= 0 && yi < a.H && xi >= 0 && xi < a.W)
-          s = a.src[((int64_t)c * a.batch + b) * a.H * a.W + (int64_t)yi * a.W + xi];
-      }
-      v[j] = s;
-    }
-    *reinterpret_cast<uint4*>(a.cols + p * a.Kp + kg * 8) = *reinterpret_cast<const uint4*>(v);
+// Sums over each half (four warps) of a 256-thread block, FP64 across the warps: out[n] by the
+// half's thread n. half_sums' out is the half's own.
+template <int N>
+__device__ __forceinline__ void half_sums(Sum (&v)[N], double* out) {
+  __shared__ double sh[8][N];
+  const int warp = threadIdx.x >> 5, t = threadIdx.x & 127;
+  warp_sums<N>(v, sh[warp]);
+  __syncthreads();
+  if (t < N) {
+    double s = 0.0;
+    for (int w = warp & 4; w < (warp & 4) + 4; ++w) s += sh[w][t];
+    out[t] = s;
   }
 }
-
-// The same with 8 channels per thread (C a multiple of 8, Kp = 9 C).
-__global__ void im2col_bf16_c8_kernel(const Im2colBf16Args a) {
-  const int cg_n = a.C / 8;
-  const int64_t P = (int64_t)a.batch * a.H * a.W;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < P * cg_n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = t % P;
-    const int cg = (int)(t / P);
-    const int x = (int)(p % a.W);
-    const int y = (int)((p / a.W) % a.H);
-    const int b = (int)(p / ((int64_t)a.W * a.H));
-    __align__(16) __nv_bfloat16 v[72];
-#pragma unroll
-    for (int cc = 0; cc < 8; ++cc) {
-      const __nv_bfloat16* s = a.src + ((int64_t)(cg * 8 + cc) * a.batch + b) * a.H * a.W;
-#pragma unroll
-      for (int tap = 0; tap < 9; ++tap) {
-        const int yi = y + tap / 3 - 1, xi = x + tap % 3 - 1;
-        v[cc * 9 + tap] = (yi >= 0 && yi < a.H && xi >= 0 && xi < a.W)
-                              ? s[(int64_t)yi * a.W + xi]
-                              : __float2bfloat16_rn(0.f);
-      }
-    }
-    uint4* dst = reinterpret_cast<uint4*>(a.cols + p * a.Kp + cg * 72);
-#pragma unroll
-    for (int q = 0; q < 9; ++q) dst[q] = reinterpret_cast<const uint4*>(v)[q];
-  }
-}
-
-__global__ void weights_t_bf16_kernel(const float* w, int cout, int cin, int Kp2,
-                                      __nv_bfloat16* wt) {
-  const int64_t n = (int64_t)cin * Kp2;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(t / Kp2), k = (int)(t % Kp2);
-    float v = 0.f;
-    if (k < 9 * cout) {
-      const int o = k / 9, tap = k - 9 * o;
-      v = w[(int64_t)o * 9 * cin + c * 9 + (8 - tap)];
-    }
-    wt[t] = __float2bfloat16_rn(v);
-  }
-}
-
-__global__ void route_grad_kernel(const RouteArgs a) {
-  const int64_t hw = (int64_t)a.H * a.W;
-  const int Hs = a.up ? a.H / 2 : a.H, Ws = a.up ? a.W / 2 : a.W;
-  const int64_t n1 = (int64_t)a.cu * a.batch * Hs * Ws, n2 = (int64_t)a.cs * a.batch * hw;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n1 + n2;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    if (t < n1) {
-      const int xs = (int)(t % Ws);
-      const int ys = (int)((t / Ws) % Hs);
-      const int64_t cb = t / ((int64_t)Ws * Hs);  // c * batch + b
-      const float* d = a.dx + cb * hw;
-      float s;
-      if (a.up) {
-        const int64_t r0 = (int64_t)(2 * ys) * a.W + 2 * xs;
-        s = d[r0];
-        s += d[r0 + 1];
-        s += d[r0 + a.W];
-        s += d[r0 + a.W + 1];
-      } else {
-        s = d[(int64_t)ys * a.W + xs];
-      }
-      if (a.acc1) a.dsrc1[t] += s;
-      else a.dsrc1[t] = s;
-    } else {
-      const int64_t u = t - n1;
-      const float s = a.dx[(int64_t)a.cu * a.batch * hw + u];
-      if (a.acc2) a.dsrc2[u] += s;
-      else a.dsrc2[u] = s;
-    }
-  }
-}
-
-// ---- col2im (gather) ------------------------------------------------------------------------
-// One thread per element of the source: the sum over its (1 or 4) positions in the input grid
-// and over the 3 x 3 taps of the output pixels that read it, in a fixed order.
-__global__ void col2im_kernel(const Col2imArgs a) {
-  const int Hs = a.up ? a.H / 2 : a.H, Ws = a.up ? a.W / 2 : a.W;
-  const int64_t n = (int64_t)a.C * a.batch * Hs * Ws;
-  const int64_t P = (int64_t)a.batch * a.Ho * a.Wo;  // rows of dcols' columns
-  const int rep = a.up ? 2 : 1;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int xs = (int)(t % Ws);
-    const int ys = (int)((t / Ws) % Hs);
-    const int64_t cb = t / ((int64_t)Ws * Hs);
-    const int b = (int)(cb % a.batch);
-    const int c = (int)(cb / a.batch);
-    const int cin = a.c_lo + c;
-    float sum = 0.f;
-    for (int dy = 0; dy < rep; ++dy)
-      for (int dx = 0; dx < rep; ++dx) {
-        const int yi = ys * rep + dy, xi = xs * rep + dx;
-#pragma unroll
-        for (int ky = 0; ky < 3; ++ky) {
-          const int ny = yi + 1 - ky;  // = stride * yo
-          if (ny < 0 || ny % a.stride) continue;
-          const int yo = ny / a.stride;
-          if (yo >= a.Ho) continue;
-#pragma unroll
-          for (int kx = 0; kx < 3; ++kx) {
-            const int nxx = xi + 1 - kx;
-            if (nxx < 0 || nxx % a.stride) continue;
-            const int xo = nxx / a.stride;
-            if (xo >= a.Wo) continue;
-            const int64_t p = ((int64_t)b * a.Ho + yo) * a.Wo + xo;
-            sum += a.dcols[(int64_t)(cin * 9 + ky * 3 + kx) * P + p];
-          }
-        }
-      }
-    if (a.accumulate)
-      a.dsrc[t] += sum;
-    else
-      a.dsrc[t] = sum;
+// Sums over the block, out[n] from thread n.
+template <int N>
+__device__ __forceinline__ void block_sums(Sum (&v)[N], double* out) {
+  __shared__ double sh[8][N];
+  warp_sums<N>(v, sh[threadIdx.x >> 5]);
+  __syncthreads();
+  if (threadIdx.x < N) {
+    double s = 0.0;
+    for (int w = 0; w < 8; ++w) s += sh[w][threadIdx.x];
+    out[threadIdx.x] = s;
   }
 }
 
 // ---- backward of act(film(pre)) ---------------------------------------------------------------
-// One block per (channel, sample).
-__global__ void act_backward_kernel(const ActBwdArgs a) {
-  __shared__ double sh[8][3];
-  const int o = blockIdx.x, b = blockIdx.y;
+// Block = (eight channels, a chunk of a sample's pixels): its lower half takes the first four
+// channels of every pixel, the upper half the others, so that a thread's sums and loads fit 64
+// registers (four blocks per SM). A thread reads four planar values of pre and dy each (coalesced
+// over the threads) and writes 8 bytes of the pixel's group. Bound by memory (10 B per value) and
+// the arithmetic of SiLU's derivative together; with one block per (channel, sample) the
+// 16-channel layers of 256 x 256 ran 256 blocks of scalar loads (161 us at batch 16, where their
+// 168 MB take 25 us), now 39 us.
+template <bool FILM>
+__global__ void __launch_bounds__(256, 4) act_backward_kernel(const ActBwdArgs a) {
+  pdl_wait();
+  const int groups = a.C / 8;
+  const int g = blockIdx.x % groups, chunk = blockIdx.x / groups, b = blockIdx.y;
+  const int half = threadIdx.x >> 7, t = threadIdx.x & 127;
   const int64_t P = (int64_t)a.batch * a.hw;
-  float g = 1.f, beta = 0.f;
-  if (a.film) {
-    const float* f = a.film + (int64_t)b * a.film_stride + a.film_off;
-    g = 1.f + f[o];
-    beta = f[a.C + o];
-  }
-  // per-thread sums in FP32 with Neumaier compensation (FP64 arithmetic is a small fraction of
-  // GB300's FP32 rate), then the block sum in FP64; the order is fixed, so results repeat
-  float sum[3] = {0.f, 0.f, 0.f}, cmp[3] = {0.f, 0.f, 0.f};
-  auto add = [&](int k, float x) {
-    const float t = sum[k] + x;
-    cmp[k] += fabsf(sum[k]) >= fabsf(x) ? (sum[k] - t) + x : (x - t) + sum[k];
-    sum[k] = t;
-  };
-  const int64_t base = (int64_t)o * P + (int64_t)b * a.hw;
-  for (int i = threadIdx.x; i < a.hw; i += blockDim.x) {
-    const float pre = a.pre[base + i];
-    const float dy = a.dy[base + i];
-    const float z = a.film ? g * pre + beta : pre;
-    const float dz = a.act ? dy * dsilu_f(z) : dy;
-    const float dpre = a.film ? dz * g : dz;
-    a.dpre[base + i] = __float2bfloat16_rn(dpre);
-    add(0, dpre);
-    add(1, dz * pre);
-    add(2, dz);
-  }
-  double acc[3];
+  const int per = (a.hw + a.chunks - 1) / a.chunks;
+  const int i1 = min(a.hw, (chunk + 1) * per);
+  const int c0 = g * 8 + half * 4;
+  float gm[4], bt[4];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) acc[k] = (double)sum[k] + (double)cmp[k];
-  block_sum<3>(acc, sh);
-  if (threadIdx.x == 0) {
-    double* out = a.partial + ((int64_t)o * a.batch + b) * 3;
-    out[0] = acc[0];
-    out[1] = acc[1];
-    out[2] = acc[2];
-  }
-}
-
-__global__ void bias_film_grad_kernel(const double* partial, int C, int batch, float* dbias,
-                                      float* dfilm, int film_stride, int film_off) {
-  for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < C; o += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < batch; ++b) {
-      const double* p = partial + ((int64_t)o * batch + b) * 3;
-      s += p[0];
-      if (dfilm) {
-        dfilm[(int64_t)b * film_stride + film_off + o] = (float)p[1];
-        dfilm[(int64_t)b * film_stride + film_off + C + o] = (float)p[2];
-      }
+  for (int j = 0; j < 4; ++j) {
+    gm[j] = 1.f;
+    bt[j] = 0.f;
+    if (FILM) {
+      const float* f = a.film + (int64_t)b * a.film_stride + a.film_off;
+      gm[j] = 1.f + f[c0 + j];
+      bt[j] = f[a.C + c0 + j];
     }
-    dbias[o] = (float)s;
   }
-}
-
-__global__ void splitk_reduce_kernel(const float* part, int splits, int64_t split_stride, int C,
-                                     int kin, int Kp, float* grad) {
-  const int64_t n = (int64_t)C * kin;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int o = (int)(t / kin), k = (int)(t % kin);
-    float s = 0.f;
-    for (int z = 0; z < splits; ++z) s += part[z * split_stride + (int64_t)o * Kp + k];
-    grad[t] = s;
-  }
-}
-
-__global__ void conv_epilogue_splitk_kernel(const float* __restrict__ part, int splits,
-                                            int64_t split_stride, int M, int N,
-                                            const ConvEpilogue e) {
-  const int64_t n = (int64_t)N * M;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int o = (int)(t / M), row = (int)(t % M);
-    float s = 0.f;
-    for (int z = 0; z < splits; ++z) s += part[z * split_stride + t];
-    const float pre = s + e.bias[o];
-    float zz = pre;
-    if (e.film) {
-      const float* f = e.film + (int64_t)(row / e.hw) * e.film_stride + e.film_off;
-      zz = (1.f + f[o]) * pre + f[N + o];
+  // sums of dz and, with FiLM, of dz pre; that of dpre is gamma times that of dz
+  constexpr int NS = FILM ? 8 : 4;
+  Sum acc[NS];
+  const float* pre_p = a.pre + (int64_t)c0 * P + (int64_t)b * a.hw;
+  const float* dy_p = a.dy + (int64_t)c0 * P + (int64_t)b * a.hw;
+  uint2* dst = reinterpret_cast<uint2*>(a.dpre) + ((int64_t)g * P + (int64_t)b * a.hw) * 2 + half;
+  for (int i = chunk * per + t; i < i1; i += 128) {
+    float pre[4], dy[4], out[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      pre[j] = __ldg(pre_p + j * P + i);
+      dy[j] = __ldg(dy_p + j * P + i);
     }
-    e.pre[t] = pre;
-    if (e.y) e.y[t] = e.act ? zz / (1.f + expf(-zz)) : zz;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float z = FILM ? gm[j] * pre[j] + bt[j] : pre[j];
+      const float dz = dy[j] * dsilu_f(z);
+      out[j] = FILM ? dz * gm[j] : dz;
+      acc[j].add(dz);
+      if constexpr (FILM) acc[4 + j].add(dz * pre[j]);
+    }
+    dst[2 * (int64_t)i] = make_uint2(pack2(out[0], out[1]), pack2(out[2], out[3]));
+  }
+  __shared__ double total[2][NS];
+  half_sums<NS>(acc, total[half]);
+  __syncthreads();
+  if (t < 4) {
+    double* o = a.sums + (((int64_t)(c0 + t) * a.batch + b) * a.chunks + chunk) * 3;
+    const double dz = total[half][t];
+    o[0] = FILM ? (double)(t == 0 ? gm[0] : t == 1 ? gm[1] : t == 2 ? gm[2] : gm[3]) * dz : dz;
+    o[1] = FILM ? total[half][4 % NS + t] : 0.0;
+    o[2] = FILM ? dz : 0.0;
   }
 }
 
-__global__ void weights_bf16_kernel(const float* w, int C, int kin, int Kp, __nv_bfloat16* wb) {
-  const int64_t n = (int64_t)C * Kp;
+__global__ void conv_epilogue_splitk_kernel(const float* __restrict__ part, int splits, int batch,
+                                            int Ho, int Wo, int N, const ConvEpilogue e) {
+  pdl_wait();
+  const int hw = Ho * Wo;
+  const int64_t P = (int64_t)batch * hw;
+  const int64_t n = (int64_t)((N + 7) / 8) * P;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
        t += (int64_t)gridDim.x * blockDim.x) {
-    const int o = (int)(t / Kp), k = (int)(t % Kp);
-    wb[t] = __float2bfloat16_rn(k < kin ? w[(int64_t)o * kin + k] : 0.f);
+    const int g = (int)(t / P);
+    const int64_t p = t - g * P;
+    const int b = (int)(p / hw), i = (int)(p - (int64_t)b * hw);
+    const float* f = e.film ? e.film + (int64_t)b * e.film_stride + e.film_off : nullptr;
+    float out[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int o = g * 8 + j;
+      out[j] = 0.f;
+      if (o >= N) continue;
+      float s = 0.f;
+      for (int z = 0; z < splits; ++z) s += part[((int64_t)z * N + o) * P + p];
+      const float pre = s + e.bias[o];
+      float zz = pre;
+      if (f) zz = (1.f + f[o]) * pre + f[N + o];
+      if (e.pre) e.pre[(int64_t)o * P + p] = pre;
+      out[j] = e.act ? zz / (1.f + expf(-zz)) : zz;
+    }
+    if (!e.y) continue;
+    store_group(e, g, b, i / Wo, i % Wo, Ho, Wo,
+                make_uint4(pack2(out[0], out[1]), pack2(out[2], out[3]), pack2(out[4], out[5]),
+                           pack2(out[6], out[7])));
   }
 }
 
@@ -463,26 +294,42 @@ __device__ __forceinline__ float base_of(int ch, float phi0) {
   return ch == 3 ? phi0 : (ch == 4 ? 1.f - phi0 : 0.f);
 }
 
-__global__ void loss_kernel(const LossArgs a) {
+// One thread per pixel, all five channels: the gradient goes straight to the output layer's dpre.
+__global__ void __launch_bounds__(256) loss_kernel(const LossArgs a) {
   __shared__ double sh[8][1];
+  const int chunk = blockIdx.x, b = blockIdx.y;
   const int64_t P = (int64_t)a.batch * a.hw;
   const int64_t n = kFields * P;
   const float inv_n2 = (float)(2.0 / (double)n);
+  const int per = (a.hw + a.chunks - 1) / a.chunks;
+  const int i1 = min(a.hw, (chunk + 1) * per);
+  const float phi0 = a.cond[3 * b + 1];
   double acc[1] = {0.0};
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int ch = (int)(t / P);
-    const int64_t p = t % P;
-    const int b = (int)(p / a.hw);
-    const int64_t i = p % a.hw;
-    const float F = a.target[((int64_t)b * kFields + ch) * a.hw + i];
-    const float tgt = (F - base_of(ch, a.cond[3 * b + 1]) - a.norm[ch]) / a.norm[kFields + ch];
-    const float d = a.out[t] - tgt;
-    a.dout[t] = inv_n2 * d;
-    acc[0] += (double)d * (double)d;
+  Sum grad[kFields];
+  uint4* dst = reinterpret_cast<uint4*>(a.dpre) + (int64_t)b * a.hw;
+  for (int i = chunk * per + threadIdx.x; i < i1; i += blockDim.x) {
+    float o[kFields];
+#pragma unroll
+    for (int ch = 0; ch < kFields; ++ch) {
+      const float F = a.target[((int64_t)b * kFields + ch) * a.hw + i];
+      const float tgt = (F - base_of(ch, phi0) - a.norm[ch]) / a.norm[kFields + ch];
+      const float d = a.out[ch * P + (int64_t)b * a.hw + i] - tgt;
+      o[ch] = inv_n2 * d;
+      acc[0] += (double)d * (double)d;
+      grad[ch].add(o[ch]);
+    }
+    dst[i] = make_uint4(pack2(o[0], o[1]), pack2(o[2], o[3]), pack2(o[4], 0.f), 0u);
   }
   block_sum<1>(acc, sh);
-  if (threadIdx.x == 0) a.partial[blockIdx.x] = acc[0] / (double)n;
+  if (threadIdx.x == 0) a.partial[(int64_t)b * a.chunks + chunk] = acc[0] / (double)n;
+  __shared__ double total[kFields];
+  block_sums<kFields>(grad, total);
+  __syncthreads();
+  if (threadIdx.x < kFields) {
+    double* s = a.sums + (((int64_t)threadIdx.x * a.batch + b) * a.chunks + chunk) * 3;
+    s[0] = total[threadIdx.x];
+    s[1] = s[2] = 0.0;
+  }
 }
 
 __global__ void sum_partials_kernel(const double* partial, int n, double* out) {
@@ -506,18 +353,13 @@ __global__ void adam_kernel(float* p, const float* g, float* m, float* v, int64_
   }
 }
 
-__global__ void geometry_kernel(float* X, int batch, int ny, int nx) {
-  const int64_t hw = (int64_t)ny * nx, P = batch * hw;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < P;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = t % hw;
-    const int x = (int)(i % nx), y = (int)(i / nx);
+__global__ void geometry_kernel(uint4* X, int ny, int nx) {
+  const int hw = ny * nx;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < hw; i += gridDim.x * blockDim.x) {
+    const int x = i % nx, y = i / nx;
     const float xi = ((float)x + 0.5f) / (float)nx - 0.5f;
     const float eta = ((float)y + 0.5f) / (float)ny - 0.5f;
-    X[t] = 1.f;
-    X[P + t] = xi;
-    X[2 * P + t] = eta;
-    X[3 * P + t] = 4.f * xi * eta;
+    X[i] = make_uint4(pack2(1.f, xi), pack2(eta, 4.f * xi * eta), 0u, 0u);
   }
 }
 
@@ -622,80 +464,38 @@ cudaError_t launch_uniform_fill(float* p, int64_t n, float scale, uint64_t seed,
   return cudaGetLastError();
 }
 
-cudaError_t launch_im2col(const Im2colArgs& a, cudaStream_t st) {
-  const int cin = a.cu + a.cs;
-  if (a.cu % 8 == 0 && cin % 8 == 0 && a.Kp == 9 * cin) {
-    const int64_t n = (int64_t)a.batch * a.Ho * a.Wo * (cin / 8);
-    im2col_c8_kernel<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(a);
-    return cudaGetLastError();
-  }
-  const int64_t n = (int64_t)a.batch * a.Ho * a.Wo * (a.Kp / 8);
-  im2col_kernel<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(a);
-  return cudaGetLastError();
+int act_chunks(int C, int batch, int hw) {
+  const int groups = std::max(1, C / 8);
+  return std::max(1, std::min((hw + 1023) / 1024, 608 / (groups * batch)));
 }
 
-cudaError_t launch_im2col_bf16(const Im2colBf16Args& a, cudaStream_t st) {
-  if (a.C % 8 == 0 && a.Kp == 9 * a.C) {
-    const int64_t n = (int64_t)a.batch * a.H * a.W * (a.C / 8);
-    im2col_bf16_c8_kernel<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(a);
-    return cudaGetLastError();
-  }
-  const int64_t n = (int64_t)a.batch * a.H * a.W * (a.Kp / 8);
-  im2col_bf16_kernel<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(a);
-  return cudaGetLastError();
+namespace {
+template <class K, class... A>
+cudaError_t launch_pdl(K kernel, dim3 grid, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
-
-cudaError_t launch_weights_t_bf16(const float* w, int cout, int cin, int Kp2, __nv_bfloat16* wt,
-                                  cudaStream_t st) {
-  weights_t_bf16_kernel<<<grid_for((int64_t)cin * Kp2, 256, 1024), 256, 0, st>>>(w, cout, cin,
-                                                                                  Kp2, wt);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_route_grad(const RouteArgs& a, cudaStream_t st) {
-  const int Hs = a.up ? a.H / 2 : a.H, Ws = a.up ? a.W / 2 : a.W;
-  const int64_t n = (int64_t)a.cu * a.batch * Hs * Ws + (int64_t)a.cs * a.batch * a.H * a.W;
-  route_grad_kernel<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_col2im(const Col2imArgs& a, cudaStream_t st) {
-  const int Hs = a.up ? a.H / 2 : a.H, Ws = a.up ? a.W / 2 : a.W;
-  const int64_t n = (int64_t)a.C * a.batch * Hs * Ws;
-  col2im_kernel<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(a);
-  return cudaGetLastError();
-}
+}  // namespace
 
 cudaError_t launch_act_backward(const ActBwdArgs& a, cudaStream_t st) {
-  act_backward_kernel<<<dim3(a.C, a.batch), 256, 0, st>>>(a);
-  return cudaGetLastError();
+  const dim3 grid(a.C / 8 * a.chunks, a.batch);
+  return a.film ? launch_pdl(act_backward_kernel<true>, grid, st, a)
+                : launch_pdl(act_backward_kernel<false>, grid, st, a);
 }
 
-cudaError_t launch_bias_film_grad(const double* partial, int C, int batch, float* dbias,
-                                  float* dfilm, int film_stride, int film_off, cudaStream_t st) {
-  bias_film_grad_kernel<<<grid_for(C, 128, 64), 128, 0, st>>>(partial, C, batch, dbias, dfilm,
-                                                              film_stride, film_off);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_splitk_reduce(const float* part, int splits, int64_t split_stride, int C,
-                                 int kin, int Kp, float* grad, cudaStream_t st) {
-  splitk_reduce_kernel<<<grid_for((int64_t)C * kin, 256, 1024), 256, 0, st>>>(
-      part, splits, split_stride, C, kin, Kp, grad);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_conv_epilogue_splitk(const float* part, int splits, int64_t split_stride,
-                                        int M, int N, const ConvEpilogue& e, cudaStream_t st) {
-  conv_epilogue_splitk_kernel<<<grid_for((int64_t)N * M, 256, 2048), 256, 0, st>>>(
-      part, splits, split_stride, M, N, e);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_weights_bf16(const float* w, int C, int kin, int Kp, __nv_bfloat16* wb,
-                                cudaStream_t st) {
-  weights_bf16_kernel<<<grid_for((int64_t)C * Kp, 256, 1024), 256, 0, st>>>(w, C, kin, Kp, wb);
-  return cudaGetLastError();
+cudaError_t launch_conv_epilogue_splitk(const float* part, int splits, int batch, int Ho, int Wo,
+                                        int N, const ConvEpilogue& e, cudaStream_t st) {
+  const int64_t n = (int64_t)((N + 7) / 8) * batch * Ho * Wo;
+  return launch_pdl(conv_epilogue_splitk_kernel, dim3(grid_for(n, 256, 2048)), st, part, splits,
+                    batch, Ho, Wo, N, e);
 }
 
 cudaError_t launch_mlp_forward(const MlpArgs& a, cudaStream_t st) {
@@ -715,7 +515,7 @@ cudaError_t launch_mlp_backward(const MlpArgs& a, const float* dr, float* gW1, f
 }
 
 cudaError_t launch_loss(const LossArgs& a, cudaStream_t st) {
-  loss_kernel<<<a.blocks, 256, 0, st>>>(a);
+  loss_kernel<<<dim3(a.chunks, a.batch), 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -730,9 +530,9 @@ cudaError_t launch_adam(float* p, const float* g, float* m, float* v, int64_t n,
   return cudaGetLastError();
 }
 
-cudaError_t launch_geometry(float* X, int batch, int ny, int nx, cudaStream_t st) {
-  geometry_kernel<<<grid_for((int64_t)batch * ny * nx, 256, 2048), 256, 0, st>>>(X, batch, ny,
-                                                                                  nx);
+cudaError_t launch_geometry(__nv_bfloat16* X, int ny, int nx, cudaStream_t st) {
+  geometry_kernel<<<grid_for((int64_t)ny * nx, 256, 2048), 256, 0, st>>>(
+      reinterpret_cast<uint4*>(X), ny, nx);
   return cudaGetLastError();
 }
 
