@@ -29,6 +29,7 @@ struct GemmArgs {
   int64_t k_per_split;  // multiple of 64
   float* d;
   int64_t ldd, split_stride;
+  int d_vec;  // set by launch_gemm: 16-byte stores of D
   int* err;  // bit 0 set when a bounded wait gave up (may be null)
   int splits;  // set by launch_gemm: K splits (tiles of D are m x n x split)
 };
