@@ -408,16 +408,16 @@ bool plan_backward(mclbm_net* n, int batch) {
     a.part = y.part;
     a.err = n->err;
     WgradMaps& m = n->wg_maps[l];
-    if (!encode_groups(&m.a, y.dpre, y.og, P, batch, y.Ho, y.Wo, 8, a.go, 16)) return false;
+    if (!encode_groups(&m.a, y.dpre, y.og, P, batch, y.Ho, y.Wo, 16, a.go, 8)) return false;
     const Input in = input_of(n, l, batch);
     const int images = l == 0 ? 1 : batch;
     if (y.stride == 1) {
-      if (!encode_groups(&m.b[0], in.x, y.groups, in.group, images, y.H, y.W, 10, a.gc, 18))
+      if (!encode_groups(&m.b[0], in.x, y.groups, in.group, images, y.H, y.W, 18, a.gc, 10))
         return false;
     } else {
       for (int p = 0; p < 4; ++p)
-        if (!encode_parity(&m.b[p], in.x, p >> 1, p & 1, y.groups, in.group, images, y.H, y.W, 9,
-                           a.gc, 17))
+        if (!encode_parity(&m.b[p], in.x, p >> 1, p & 1, y.groups, in.group, images, y.H, y.W, 17,
+                           a.gc, 9))
           return false;
       if (!encode_groups(&n->dx_map[l], y.dpre, y.og, P, batch, y.Ho, y.Wo, 9,
                          dx_stride2_kg(y.cout), 17))

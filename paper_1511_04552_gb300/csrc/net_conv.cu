@@ -649,9 +649,9 @@ __global__ void __launch_bounds__(kS2Threads) dx_stride2_kernel(
 
 // ---- weight gradient ------------------------------------------------------------------------
 // dW[o][c][tap] = sum over pixels of dpre[o][pixel] x[c][pixel + tap]: M = o, K = pixels, N =
-// (tap, channel). A stage holds one tile of 16 rows x 8 pixels of dpre and the patch of x its taps
-// read, both by TMA in the MN-major core-matrix layout (8 pixels x 16 bytes), rows of a patch
-// ordered [y][group][x]: the groups of one row and those of the next follow each other at one
+// (tap, channel). A stage holds one tile of 8 rows x 16 pixels of dpre and the patch of x its taps
+// read, both by TMA in the MN-major core-matrix layout (8 pixels x 16 bytes; a K step is one row of
+// 16 pixels), rows of a patch ordered [y][group][x]: the groups of one row and those of the next follow each other at one
 // stride, so that one MMA takes the three vertical taps of all groups (N = 24 groups' columns) and
 // a horizontal tap is a start address 16 bytes on. The stride-2 layers read x as four parity
 // patches (TMA with a pixel stride of 2). One CTA per (split of the pixel tiles, channel chunk,
@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(kWgThreads) wgrad_kernel(
         break;
       }
       if (leader) {
-        const int y0 = ty * 16, x0 = tx * 8;
+        const int y0 = ty * kTileH, x0 = tx * kTileW;
         const uint32_t fb = smem_addr(&full[st]), sa = smem_addr(smem + st * a.stage_bytes);
         bar_expect_tx(fb, (uint32_t)a.tx_bytes);
         tma_load_4d(sa, &maps.a, x0 * 8, oc * a.go, y0, b, fb);
@@ -742,9 +742,8 @@ __global__ void __launch_bounds__(kWgThreads) wgrad_kernel(
       e_off[e] = (uint32_t)w.off >> 4;
       e_desc[e] = instr_desc(kRows, w.n, true, true);
     }
-    const uint32_t a_row = (uint32_t)a.go * 128;
-    const uint32_t a_two = a_row >> 3, b_two = (uint32_t)a.b_row >> 3;  // two rows, 16-byte units
-    const uint32_t hi_a = desc_hi(128), hi_b = desc_hi((uint32_t)a.b_group);
+    const uint32_t a_row = (uint32_t)a.go * kTileW, b_row = (uint32_t)a.b_row >> 4;  // 16 bytes
+    const uint32_t hi_a = desc_hi(kTileW * 16), hi_b = desc_hi((uint32_t)a.b_group);
     int st = 0;
     uint32_t round = 0;
     for (int t = t0; t < t1 && !*abort; ++t, ++mma_done) {
@@ -754,13 +753,13 @@ __global__ void __launch_bounds__(kWgThreads) wgrad_kernel(
       }
       tc_fence_after();
       const uint32_t sa = smem_addr(smem + st * a.stage_bytes);
-      const uint32_t a_lo = desc_lo(sa, a_row), b_lo = desc_lo(sa + a.a_bytes, (uint32_t)a.b_row);
+      const uint32_t a_lo = desc_lo(sa, 128), b_lo = desc_lo(sa + a.a_bytes, 128);
 #pragma unroll
       for (int e = 0; e < 6; ++e) {
         if (e >= a.entries) break;
 #pragma unroll
-        for (uint32_t ks = 0; ks < 8; ++ks)  // 16 pixels: two rows of the tile
-          mma_bf16_words(leader, d_col[e], a_lo + ks * a_two, hi_a, b_lo + e_off[e] + ks * b_two,
+        for (uint32_t ks = 0; ks < kTileH; ++ks)
+          mma_bf16_words(leader, d_col[e], a_lo + ks * a_row, hi_a, b_lo + e_off[e] + ks * b_row,
                          hi_b, e_desc[e], ks > 0 ? 1u : accumulate);
       }
       accumulate = 1;
@@ -1042,21 +1041,18 @@ void wgrad_chunk(WgradArgs* a, int cin_groups, int chunks) {
   auto r16 = [](int n) { return (n + 15) / 16 * 16; };
   a->chunks = chunks;
   a->gc = (cin_groups + chunks - 1) / chunks;
+  const int px = a->s2 ? kTileW + 1 : kTileW + 2, rows = a->s2 ? kTileH + 1 : kTileH + 2;
+  const int patches = a->s2 ? 4 : 1;
+  a->b_group = px * 16;
+  a->b_row = a->gc * a->b_group;
+  a->patch_bytes = (rows * a->b_row + 127) / 128 * 128;
+  a->tx_bytes = a->a_bytes + patches * rows * a->b_row;
+  a->stage_bytes = a->a_bytes + patches * a->patch_bytes;
   if (!a->s2) {
-    a->b_group = 10 * 16;
-    a->b_row = a->gc * a->b_group;
-    a->patch_bytes = (18 * a->b_row + 127) / 128 * 128;
-    a->tx_bytes = a->a_bytes + 18 * a->b_row;
-    a->stage_bytes = a->a_bytes + a->patch_bytes;
     const int n = r16(24 * a->gc);
     for (int dx = 0; dx < 3; ++dx) a->e[dx] = {dx * 16, n, dx * n};
     a->cols = 3 * n;
   } else {
-    a->b_group = kS2Px * 16;
-    a->b_row = a->gc * a->b_group;
-    a->patch_bytes = (kS2Rows * a->b_row + 127) / 128 * 128;
-    a->tx_bytes = a->a_bytes + 4 * kS2Rows * a->b_row;
-    a->stage_bytes = a->a_bytes + 4 * a->patch_bytes;
     // kx = 0 and 2 read the odd columns (x - 1 and x of their patch), kx = 1 the even ones; ky
     // likewise: odd rows hold ky = 0 and, one row on, ky = 2
     const int n2 = r16(16 * a->gc), n1 = r16(8 * a->gc);
@@ -1085,20 +1081,20 @@ void wgrad_rows(WgradArgs* a, int cout, int stride) {
   a->go = std::min(16, og);
   a->ochunks = (og + 15) / 16;
   a->mrows = std::min(kRows, og * 8);
-  a->a_bytes = 16 * a->go * 128;
+  a->a_bytes = kTileH * a->go * kTileW * 16;
 }
 
 }  // namespace
 
 // Splits x channel chunks x parts (the horizontal taps apart, or together) CTAs: the splits are
 // fixed by the accuracy, the rest is chosen for the least estimated time. An MMA of N columns
-// takes max(32, N / 2) cycles (its A operand, 4 KiB, is read at 128 B per cycle), a tile is also
-// bound by its bytes, and CTAs beyond one per SM share it.
+// takes max(45, N / 2) cycles (measured), a tile is also bound by its bytes, and CTAs beyond one
+// per SM share it.
 void plan_wgrad(WgradArgs* a, int cin_groups, int cout, int kin, int Ho, int Wo, int batch,
                 int stride, int sms) {
   wgrad_rows(a, cout, stride);
-  a->tiles_x = (Wo + 7) / 8;
-  a->tiles_y = (Ho + 15) / 16;
+  a->tiles_x = (Wo + kTileW - 1) / kTileW;
+  a->tiles_y = (Ho + kTileH - 1) / kTileH;
   a->batch = batch;
   const int tiles = a->tiles_x * a->tiles_y * batch;
   a->split_tiles = (tiles + wgrad_splits(cout, kin) - 1) / wgrad_splits(cout, kin);
@@ -1110,7 +1106,7 @@ void plan_wgrad(WgradArgs* a, int cin_groups, int cout, int kin, int Ho, int Wo,
     wgrad_chunk(a, cin_groups, (cin_groups + gc - 1) / gc);
     for (int parts = 1; parts <= taps; parts *= 3) {
       double mma = 0.0;
-      for (int e = 0; e < taps / parts; ++e) mma += std::max(32, a->e[e].n / 2);
+      for (int e = 0; e < taps / parts; ++e) mma += std::max(45, a->e[e].n / 2);
       const double tile = std::max(8.0 * mma, a->tx_bytes / 40.0);
       const double ctas = (double)a->splits * a->chunks * a->ochunks * parts;
       const double t = tile * a->split_tiles * std::max(1.0, ctas / sms);
