@@ -49,6 +49,13 @@ struct mclbm {
 
 namespace {
 
+// Steps per launch of the cluster-resident kernel: it costs a launch, a load and a store of the
+// state, so calls of few steps go to the step-by-step kernels (4 steps: 32 x 32 10 us against 22,
+// 130 x 67 23 against 20; 8 steps: 14 against 39, 35 against 35); long ones are cut into launches of
+// 2^14 (a multiple of the largest block of stochastic-rounding seeds).
+constexpr int64_t kClusterMaxSteps = 1 << 14;
+int64_t cluster_min_steps(const StepConfig& c) { return c.cl_threads <= 512 ? 4 : 8; }
+
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 int fail(mclbm_t* h, int code, const char* fmt, ...) {
@@ -292,10 +299,19 @@ int mclbm_bind(mclbm_t* h, void* dev_buf, size_t bytes, void* cuda_stream) {
       h->cfg.variant = 0;
     }
   }
+  // small lattices: several steps per launch in one cluster, unless a step kernel is asked for by
+  // the MCLBM_STEP_* variables (MCLBM_STEP_VARIANT = cluster asks for this one)
+  const char* sv = std::getenv("MCLBM_STEP_VARIANT");
+  if ((!sv || std::strcmp(sv, "cluster") == 0) && !std::getenv("MCLBM_STEP_VEC") &&
+      !std::getenv("MCLBM_STEP_TILE_H") &&
+      prepare_cluster(&h->cfg, h->L, h->k.mask == MCLBM_F_ALL && !h->k.two_sets,
+                      h->k.two_sets != 0) != cudaSuccess) {
+    cudaGetLastError();
+    h->cfg.cl_ctas = 0;
+  }
   // MCLBM_STEP_VARIANT = two (FP32 lattices of at most one 32 x 16 tile per SM): pairs of steps
   // in one launch, bitwise the same states; not the default, since it is no faster (the first
   // step's 1.7x redundant work outweighs the launch it saves)
-  const char* sv = std::getenv("MCLBM_STEP_VARIANT");
   const bool two_asked = sv && std::strcmp(sv, "two") == 0;
   if (two_asked && h->cfg.variant == 2 && h->L.storage == MCLBM_STORE_F32 &&
       h->L.np == kPlanes && h->cfg.vec != 2) {
@@ -336,9 +352,20 @@ int mclbm_step(mclbm_t* h, int64_t n) {
   int rc = ready(h, true);
   if (rc) return rc;
   if (n < 0) return fail(h, MCLBM_EINVAL, "negative step count");
+  // small lattices: the whole call in launches of the cluster-resident kernel
+  int64_t left = n;
+  while (h->cfg.cl_ctas > 0 && left >= cluster_min_steps(h->cfg)) {
+    const int64_t m = left < kClusterMaxSteps ? left : kClusterMaxSteps;
+    StepArgs a = step_args(h, h->cur, 0);
+    const int to = h->cur ^ (int)(m & 1);
+    a.dst = h->state[to];
+    CK(h, launch_cluster(a, h->cfg, (int)m, (uint32_t)h->steps, h->epoch, h->stream));
+    h->cur = to;
+    h->steps += m;
+    left -= m;
+  }
   // the even part in graphs of 2^k steps, largest first (1000 = 512 + 256 + 128 + 64 + 32 + 8;
   // each graph boundary costs about 4 us of idle GPU), an odd last step as a single launch
-  int64_t left = n;
   while (left >= 2) {
     int k = 1;
     while (k < kGraphLogMax && (int64_t(2) << k) <= left) ++k;

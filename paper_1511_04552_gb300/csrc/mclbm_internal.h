@@ -87,6 +87,9 @@ struct StepConfig {
   bool two;     // FP32: pairs of steps by the two-step kernel (set by prepare_two_f32)
   int grid2;    // two-step kernel: CTAs (one per 32 x 16 tile)
   int th;       // TMA kernel: tile height, 8 or 7 (0 before prepare_step: chosen by lattice)
+  // cluster-resident kernel (mclbm_cluster.cuh), set by prepare_cluster: CTAs of the cluster (0: not
+  // used), nodes and threads of each
+  int cl_ctas, cl_run, cl_threads;
 };
 StepConfig choose_step_config(int nx, int ny, int np);
 // Device-dependent set-up of the chosen variant (shared-memory limit, persistent grid size);
@@ -104,6 +107,20 @@ cudaError_t make_two_step_tensor_map(CUtensorMap* map, void* state0, const Layou
 cudaError_t prepare_two_f32(StepConfig* c, const Layout& L);
 cudaError_t launch_two_f32(const StepArgs& a, const StepConfig& c, const CUtensorMap* map2,
                            cudaStream_t st);
+// Cluster-resident kernel: enables it in c where the lattice fits one cluster; n steps in one launch
+// from a.src to a.dst.
+cudaError_t prepare_cluster(StepConfig* c, const Layout& L, bool all, bool two);
+cudaError_t launch_cluster(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
+                           uint32_t* epoch, cudaStream_t st);
+cudaError_t prepare_cluster_f32(StepConfig* c, const Layout& L, bool all, bool two);
+cudaError_t prepare_cluster_f16(StepConfig* c, const Layout& L, bool all, bool two);
+cudaError_t prepare_cluster_bf16(StepConfig* c, const Layout& L, bool all, bool two);
+cudaError_t launch_cluster_f32(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
+                               uint32_t* epoch, cudaStream_t st);
+cudaError_t launch_cluster_f16(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
+                               uint32_t* epoch, cudaStream_t st);
+cudaError_t launch_cluster_bf16(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
+                                uint32_t* epoch, cudaStream_t st);
 // Tile width of a configured step kernel's TMA maps.
 int step_tile_width(const StepConfig& c);
 cudaError_t launch_step(const StepArgs& a, const StepConfig& c, const CUtensorMap* map,

@@ -1,5 +1,8 @@
 // Step kernels of libmclbm for state storage type __nv_bfloat16 (one translation unit per storage
 // type, so the build compiles them in parallel).
+#include <algorithm>
+
+#include "mclbm_cluster.cuh"
 #include "mclbm_pair.cuh"
 
 namespace mcl {
@@ -11,6 +14,15 @@ cudaError_t launch_step_bf16(const StepArgs& a, const StepConfig& c, const CUten
 
 cudaError_t prepare_tma_bf16(StepConfig* c, const Layout& L) {
   return pair::prepare_pair_tma_t<__nv_bfloat16>(c, L);
+}
+
+cudaError_t prepare_cluster_bf16(StepConfig* c, const Layout& L, bool all, bool two) {
+  return cluster::prepare<__nv_bfloat16>(c, L, all, two);
+}
+
+cudaError_t launch_cluster_bf16(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
+                              uint32_t* epoch, cudaStream_t st) {
+  return cluster::launch<__nv_bfloat16>(a, c, n, steps0, epoch, st);
 }
 
 }  // namespace mcl

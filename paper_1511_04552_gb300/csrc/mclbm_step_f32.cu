@@ -1,5 +1,8 @@
 // Step kernels of libmclbm for state storage type float (one translation unit per storage
 // type, so the build compiles them in parallel).
+#include <algorithm>
+
+#include "mclbm_cluster.cuh"
 #include "mclbm_pair.cuh"
 #include "mclbm_pair2.cuh"
 
@@ -19,6 +22,15 @@ cudaError_t prepare_two_f32(StepConfig* c, const Layout& L) { return pair::prepa
 cudaError_t launch_two_f32(const StepArgs& a, const StepConfig& c, const CUtensorMap* map2,
                            cudaStream_t st) {
   return pair::launch_two(a, c, map2, st);
+}
+
+cudaError_t prepare_cluster_f32(StepConfig* c, const Layout& L, bool all, bool two) {
+  return cluster::prepare<float>(c, L, all, two);
+}
+
+cudaError_t launch_cluster_f32(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
+                              uint32_t* epoch, cudaStream_t st) {
+  return cluster::launch<float>(a, c, n, steps0, epoch, st);
 }
 
 }  // namespace mcl
