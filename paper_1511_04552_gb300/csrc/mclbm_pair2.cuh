@@ -41,6 +41,16 @@ struct SmemAcc {
   __device__ __forceinline__ float a1(int p, int dx, int dy) const {
     return base[p * WPLANE + dy * WX + dx];
   }
+  __device__ __forceinline__ int pick(bool c, int p, int dx, int dy, int other) const {
+    return c ? p * WPLANE + dy * WX + dx : other;
+  }
+  __device__ __forceinline__ int pick(bool c, int p, int dx, int dy, int p2, int dx2,
+                                      int dy2) const {
+    return pick(c, p, dx, dy, p2 * WPLANE + dy2 * WX + dx2);
+  }
+  __device__ __forceinline__ float at(int place, int planes) const {
+    return base[place + planes * WPLANE];
+  }
   __device__ __forceinline__ float2 a2(int p, int dy) const {
     return *reinterpret_cast<const float2*>(base + p * WPLANE + dy * WX);
   }
