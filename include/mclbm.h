@@ -159,9 +159,10 @@ int mclbm_bind(mclbm_t *h, void *dev_buf, size_t bytes, void *cuda_stream);
 int mclbm_init(mclbm_t *h, int mode, const float *warm_dev);
 
 /* Advances n >= 0 time steps (Eqs 18-19 with the forces of Table 1 and the walls of
- * Eqs 34-36). Lattices of up to about 10 000 nodes run a call of several steps in one launch (up to
- * 2^14 steps each), the cavity resident in the shared memory of one thread-block cluster; others run
- * the even part in captured CUDA graphs of 2^k steps (2 <= 2^k <= 1024, largest first, built on
+ * Eqs 34-36). Lattices of up to about 75 000 nodes run a call of several steps in one launch (up to
+ * 2^14 steps each), the cavity resident in shared memory: the small ones in one thread-block cluster,
+ * the larger ones (from 16 steps) in a cooperative grid over the device, which uses the state level
+ * that is not current as scratch; others run the even part in captured CUDA graphs of 2^k steps (2 <= 2^k <= 1024, largest first, built on
  * first use and kept with the handle) and an odd last step as a single launch, with the same states
  * bit for bit. The stochastic-rounding streams of 16-bit storage follow the graphs' replay count, so a given
  * sequence of calls is reproducible bit for bit. Async. A step kernel
@@ -350,9 +351,9 @@ int64_t mclbm_steps_done(const mclbm_t *h);
  * kernel's tile height (8, or 7 where 32 x 8 tiles would give some SMs a second tile and 32 x 7
  * tiles fit two per SM, e.g. 256 x 256 on 152 SMs; 8 for the tile kernel);
  * grid: the TMA kernel's persistent CTAs (0 for the tile kernel); two: 1 when pairs of steps run
- * in the two-step kernel. It is the kernel of single steps: calls of several steps on small
- * lattices go to the cluster-resident kernel (mclbm_step). Outputs may be NULL. Host only, no GPU work. MCLBM_EINVAL for a NULL
- * handle, MCLBM_ESTATE before mclbm_bind. */
+ * in the two-step kernel. It is the kernel of single steps: calls of several steps on lattices that
+ * fit shared memory go to the resident kernels (mclbm_step). Outputs may be NULL. Host only, no GPU
+ * work. MCLBM_EINVAL for a NULL handle, MCLBM_ESTATE before mclbm_bind. */
 int mclbm_step_kernel(const mclbm_t *h, int *variant, int *nodes_per_thread, int *tile_h,
                       int *grid, int *two);
 

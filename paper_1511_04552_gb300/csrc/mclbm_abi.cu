@@ -55,6 +55,13 @@ namespace {
 // 2^14 (a multiple of the largest block of stochastic-rounding seeds).
 constexpr int64_t kClusterMaxSteps = 1 << 14;
 int64_t cluster_min_steps(const StepConfig& c) { return c.cl_threads <= 512 ? 4 : 8; }
+// The same for the grid-resident kernel (16 steps: 128 x 128 41 us against 61, 256 x 256 75 against 74, 8
+// steps 41 for 256 x 256 step by step), in even numbers; a launch has as many steps as there are
+// CTAs along a side (mclbm_resident.cuh).
+int64_t resident_min_steps(const StepConfig& c) {
+  const int across = c.re_gx > c.re_gy ? c.re_gx : c.re_gy;
+  return across <= 16 ? 16 : (across + 1) & ~1;
+}
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -309,6 +316,18 @@ int mclbm_bind(mclbm_t* h, void* dev_buf, size_t bytes, void* cuda_stream) {
     cudaGetLastError();
     h->cfg.cl_ctas = 0;
   }
+  // larger ones, as far as the device's shared memory goes: several steps per launch in one grid
+  // (MCLBM_STEP_VARIANT = resident asks for it). The cluster keeps what gives its CTAs few nodes: per
+  // step, 64 x 64 1.52 us against 2.01 and 72 x 72 2.04 against 1.66, at 256 and 324 nodes of each CTA
+  const bool resident_asked = sv && std::strcmp(sv, "resident") == 0;
+  if (resident_asked || (!sv && !std::getenv("MCLBM_STEP_VEC") && !std::getenv("MCLBM_STEP_TILE_H") &&
+                         (h->cfg.cl_ctas == 0 || h->cfg.cl_run > 320))) {
+    if (prepare_resident(&h->cfg, h->L, h->k.mask == MCLBM_F_ALL && !h->k.two_sets,
+                         h->k.two_sets != 0) != cudaSuccess) {
+      cudaGetLastError();
+      h->cfg.re_ctas = 0;
+    }
+  }
   // MCLBM_STEP_VARIANT = two (FP32 lattices of at most one 32 x 16 tile per SM): pairs of steps
   // in one launch, bitwise the same states; not the default, since it is no faster (the first
   // step's 1.7x redundant work outweighs the launch it saves)
@@ -352,8 +371,17 @@ int mclbm_step(mclbm_t* h, int64_t n) {
   int rc = ready(h, true);
   if (rc) return rc;
   if (n < 0) return fail(h, MCLBM_EINVAL, "negative step count");
-  // small lattices: the whole call in launches of the cluster-resident kernel
   int64_t left = n;
+  // middling lattices: the even part in launches of the grid-resident kernel
+  while (h->cfg.re_ctas > 0 && left >= resident_min_steps(h->cfg)) {
+    const int64_t m = (left < kClusterMaxSteps ? left : kClusterMaxSteps) & ~int64_t(1);
+    StepArgs a = step_args(h, h->cur, 0);
+    a.dst = h->state[h->cur];
+    CK(h, launch_resident(a, h->cfg, (int)m, h->state[1 - h->cur], h->epoch, h->stream));
+    h->steps += m;
+    left -= m;
+  }
+  // small ones: the whole call in launches of the cluster-resident kernel
   while (h->cfg.cl_ctas > 0 && left >= cluster_min_steps(h->cfg)) {
     const int64_t m = left < kClusterMaxSteps ? left : kClusterMaxSteps;
     StepArgs a = step_args(h, h->cur, 0);

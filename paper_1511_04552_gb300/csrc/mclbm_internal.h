@@ -90,6 +90,9 @@ struct StepConfig {
   // cluster-resident kernel (mclbm_cluster.cuh), set by prepare_cluster: CTAs of the cluster (0: not
   // used), nodes and threads of each
   int cl_ctas, cl_run, cl_threads;
+  // grid-resident kernel (mclbm_resident.cuh), set by prepare_resident: its CTAs (0: not used), the
+  // tiles they cut the lattice into along x and y, and the threads of each
+  int re_ctas, re_gx, re_gy, re_threads;
 };
 StepConfig choose_step_config(int nx, int ny, int np);
 // Device-dependent set-up of the chosen variant (shared-memory limit, persistent grid size);
@@ -120,6 +123,20 @@ cudaError_t launch_cluster_f32(const StepArgs& a, const StepConfig& c, int n, ui
 cudaError_t launch_cluster_f16(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
                                uint32_t* epoch, cudaStream_t st);
 cudaError_t launch_cluster_bf16(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
+                                uint32_t* epoch, cudaStream_t st);
+// Grid-resident kernel: enables it in c where the lattice fits the device's shared memory; n steps
+// (even) in one launch from a.src to a.dst, the same level. scratch: the other level.
+cudaError_t prepare_resident(StepConfig* c, const Layout& L, bool all, bool two);
+cudaError_t launch_resident(const StepArgs& a, const StepConfig& c, int n, void* scratch,
+                            uint32_t* epoch, cudaStream_t st);
+cudaError_t prepare_resident_f32(StepConfig* c, const Layout& L, bool all, bool two);
+cudaError_t prepare_resident_f16(StepConfig* c, const Layout& L, bool all, bool two);
+cudaError_t prepare_resident_bf16(StepConfig* c, const Layout& L, bool all, bool two);
+cudaError_t launch_resident_f32(const StepArgs& a, const StepConfig& c, int n, void* scratch,
+                                uint32_t* epoch, cudaStream_t st);
+cudaError_t launch_resident_f16(const StepArgs& a, const StepConfig& c, int n, void* scratch,
+                                uint32_t* epoch, cudaStream_t st);
+cudaError_t launch_resident_bf16(const StepArgs& a, const StepConfig& c, int n, void* scratch,
                                 uint32_t* epoch, cudaStream_t st);
 // Tile width of a configured step kernel's TMA maps.
 int step_tile_width(const StepConfig& c);

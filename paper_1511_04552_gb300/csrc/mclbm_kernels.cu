@@ -456,6 +456,7 @@ StepConfig choose_step_config(int nx, int ny, int np) {
   c.two = false;
   c.grid2 = 0;
   c.cl_ctas = c.cl_run = c.cl_threads = 0;
+  c.re_ctas = c.re_gx = c.re_gy = c.re_threads = 0;
   // MCLBM_STEP_VEC = 1 | 2 forces the nodes per thread (comparisons; default by lattice size)
   const char* vv = std::getenv("MCLBM_STEP_VEC");
   c.vec = (vv && (vv[0] == '1' || vv[0] == '2') && vv[1] == 0) ? vv[0] - '0' : 0;
@@ -521,6 +522,33 @@ cudaError_t launch_cluster(const StepArgs& a, const StepConfig& c, int n, uint32
       return launch_cluster_f16(a, c, n, steps0, epoch, st);
     case MCLBM_STORE_BF16:
       return launch_cluster_bf16(a, c, n, steps0, epoch, st);
+    default:
+      return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t prepare_resident(StepConfig* c, const Layout& L, bool all, bool two) {
+  switch (L.storage) {
+    case MCLBM_STORE_F32:
+      return prepare_resident_f32(c, L, all, two);
+    case MCLBM_STORE_F16:
+      return prepare_resident_f16(c, L, all, two);
+    case MCLBM_STORE_BF16:
+      return prepare_resident_bf16(c, L, all, two);
+    default:
+      return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_resident(const StepArgs& a, const StepConfig& c, int n, void* scratch,
+                            uint32_t* epoch, cudaStream_t st) {
+  switch (a.L.storage) {
+    case MCLBM_STORE_F32:
+      return launch_resident_f32(a, c, n, scratch, epoch, st);
+    case MCLBM_STORE_F16:
+      return launch_resident_f16(a, c, n, scratch, epoch, st);
+    case MCLBM_STORE_BF16:
+      return launch_resident_bf16(a, c, n, scratch, epoch, st);
     default:
       return cudaErrorInvalidValue;
   }

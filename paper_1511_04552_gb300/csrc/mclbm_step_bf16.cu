@@ -4,6 +4,7 @@
 
 #include "mclbm_cluster.cuh"
 #include "mclbm_pair.cuh"
+#include "mclbm_resident.cuh"
 
 namespace mcl {
 
@@ -23,6 +24,15 @@ cudaError_t prepare_cluster_bf16(StepConfig* c, const Layout& L, bool all, bool 
 cudaError_t launch_cluster_bf16(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
                               uint32_t* epoch, cudaStream_t st) {
   return cluster::launch<__nv_bfloat16>(a, c, n, steps0, epoch, st);
+}
+
+cudaError_t prepare_resident_bf16(StepConfig* c, const Layout& L, bool all, bool two) {
+  return resident::prepare<__nv_bfloat16>(c, L, all, two);
+}
+
+cudaError_t launch_resident_bf16(const StepArgs& a, const StepConfig& c, int n, void* scratch,
+                               uint32_t* epoch, cudaStream_t st) {
+  return resident::launch<__nv_bfloat16>(a, c, n, scratch, epoch, st);
 }
 
 }  // namespace mcl

@@ -4,6 +4,7 @@
 
 #include "mclbm_cluster.cuh"
 #include "mclbm_pair.cuh"
+#include "mclbm_resident.cuh"
 #include "mclbm_pair2.cuh"
 
 namespace mcl {
@@ -31,6 +32,15 @@ cudaError_t prepare_cluster_f32(StepConfig* c, const Layout& L, bool all, bool t
 cudaError_t launch_cluster_f32(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
                               uint32_t* epoch, cudaStream_t st) {
   return cluster::launch<float>(a, c, n, steps0, epoch, st);
+}
+
+cudaError_t prepare_resident_f32(StepConfig* c, const Layout& L, bool all, bool two) {
+  return resident::prepare<float>(c, L, all, two);
+}
+
+cudaError_t launch_resident_f32(const StepArgs& a, const StepConfig& c, int n, void* scratch,
+                               uint32_t* epoch, cudaStream_t st) {
+  return resident::launch<float>(a, c, n, scratch, epoch, st);
 }
 
 }  // namespace mcl
