@@ -40,9 +40,10 @@ STEP_SOURCES = ("mclbm_device.cuh", "mclbm_pair.cuh")  # the step kernels' sourc
 
 
 def step_launches(n):
-    """Kernel launches of mclbm_step(n) on one cavity (the library's decomposition): the even
-    part in graphs of 2^k <= 1024 steps, largest first, each graph one step kernel per step and
-    one epoch kernel; an odd last step as a single launch."""
+    """Kernel launches of mclbm_step(n) on a cavity that does not fit shared memory (the library's
+    decomposition; mclbm_step_launches counts for a given cavity): the even part in graphs of
+    2^k <= 1024 steps, largest first, each graph one step kernel per step and one epoch kernel;
+    an odd last step as a single launch."""
     launches, left = 0, n
     while left >= 2:
         k = 1
@@ -358,7 +359,7 @@ def warm_start_measure(m, torch, n_points=12):
 
 
 def time_steps_only(cav, torch, nsteps):
-    """Average duration of one step launch: events around back-to-back graph replays."""
+    """Average duration of one step: events around a call of many steps."""
     st = cav.stream
     a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     cav.step(nsteps)  # warm
@@ -437,6 +438,8 @@ def main():
     hbm_peak, peak_kind = peaks()
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     achieved = bytes_lu * nx * ny / step_time / 1e9
+    launches = cav.step_launches(CH)
+    per_launch = CH if launches < CH else 1  # steps of one launch (all: state in shared memory)
 
     # end to end through the C ABI with host buffers: H2D warm fields, init, 1000 steps,
     # all 8 fields and the Nusselt numbers back to the host
@@ -501,16 +504,19 @@ def main():
                            2 * 27 * 4 * nx * ny / 1e6)},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                          "frac": achieved / hbm_peak,
-                         "traffic": ncu_traffic(w["name"]) if args.storage == "f32" else None,
+                         "traffic": ncu_traffic(w["name"])
+                                    if args.storage == "f32" and per_launch == 1 else None,
                          "peak_kind": peak_kind,
-                         "kernel": "step_pair_tma_kernel",
+                         "kernel": "step_pair_tma_kernel" if per_launch == 1 else
+                                   "step_resident_kernel",
                          "nodes_per_thread": nodes_per_thread(nx, ny, sms),
-                         "bytes_per_launch": bytes_lu * nx * ny,
-                         "launch_us": step_time * 1e6},
+                         "steps_per_launch": per_launch,
+                         "bytes_per_launch": bytes_lu * nx * ny * per_launch,
+                         "launch_us": step_time * 1e6 * per_launch},
             "e2e": {"value": e2e_value, "unit": UNIT,
                     "h2d_bytes_per_step": 4 * nx * ny * 4,
                     "d2h_bytes_per_step": 8 * nx * ny * 4 + 16},
-            "gpu_launches": args.steps * (step_launches(CH) + OUR_KERNELS_PER_REDUCTION),
+            "gpu_launches": args.steps * (launches + OUR_KERNELS_PER_REDUCTION),
             "clocks": clk.summary(),
         }
         line.update(extras)

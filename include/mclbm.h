@@ -357,6 +357,11 @@ int64_t mclbm_steps_done(const mclbm_t *h);
 int mclbm_step_kernel(const mclbm_t *h, int *variant, int *nodes_per_thread, int *tile_h,
                       int *grid, int *two);
 
+/* How many kernels mclbm_step(h, n) launches (a diagnostic): one for up to 2^14 steps where the lattice
+ * is resident in shared memory, else one per step and one per captured graph. Host only, no GPU
+ * work. -1 for a NULL or unbound handle or n < 0. */
+int64_t mclbm_step_launches(const mclbm_t *h, int64_t n);
+
 /* Text of the handle's latest error ("" if none); static text for a NULL handle. */
 const char *mclbm_last_error(const mclbm_t *h);
 

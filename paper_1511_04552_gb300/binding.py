@@ -26,7 +26,8 @@ EXPORTS = ("mclbm_props_default", "mclbm_create", "mclbm_destroy", "mclbm_buffer
            "mclbm_bind", "mclbm_init", "mclbm_step", "mclbm_stream_only", "mclbm_fields",
            "mclbm_nusselt", "mclbm_mass", "mclbm_residual", "mclbm_diagnostics",
            "mclbm_state_get", "mclbm_state_set", "mclbm_run_host", "mclbm_get_consts",
-           "mclbm_steps_done", "mclbm_step_kernel", "mclbm_last_error", "mclbm_strerror",
+           "mclbm_steps_done", "mclbm_step_kernel", "mclbm_step_launches", "mclbm_last_error",
+           "mclbm_strerror",
            "mclbm_mass_noalloc", "mclbm_save", "mclbm_load", "mclbm_selftest_wait_timeout",
            "mclbm_batch_buffer_bytes", "mclbm_batch_create", "mclbm_batch_step",
            "mclbm_batch_nusselt", "mclbm_batch_set_active", "mclbm_batch_tune",
@@ -126,6 +127,8 @@ def lib():
         ip = C.POINTER(C.c_int)
         L.mclbm_step_kernel.argtypes = [vp, ip, ip, ip, ip, ip]
         L.mclbm_step_kernel.restype = C.c_int
+        L.mclbm_step_launches.argtypes = [vp, C.c_int64]
+        L.mclbm_step_launches.restype = C.c_int64
         L.mclbm_last_error.argtypes = [vp]
         L.mclbm_last_error.restype = C.c_char_p
         L.mclbm_strerror.argtypes = [C.c_int]
@@ -296,6 +299,10 @@ class Cavity:
             raise MclbmError(rc, "mclbm_step_kernel")
         return dict(zip(("variant", "nodes_per_thread", "tile_h", "grid", "two"),
                         (x.value for x in v)))
+
+    def step_launches(self, n: int) -> int:
+        """mclbm_step_launches: kernels launched by step(n)."""
+        return int(lib().mclbm_step_launches(self._h, int(n)))
 
     # -- the C entry points
     def init(self, mode=INIT_REST, warm=None):

@@ -733,6 +733,27 @@ int mclbm_step_kernel(const mclbm_t* h, int* variant, int* nodes_per_thread, int
   return MCLBM_OK;
 }
 
+int64_t mclbm_step_launches(const mclbm_t* h, int64_t n) {
+  if (!h || !h->buf || n < 0) return -1;
+  int64_t launches = 0, left = n;
+  while (h->cfg.re_ctas > 0 && left >= resident_min_steps(h->cfg)) {
+    left -= (left < kClusterMaxSteps ? left : kClusterMaxSteps) & ~int64_t(1);
+    ++launches;
+  }
+  while (h->cfg.cl_ctas > 0 && left >= cluster_min_steps(h->cfg)) {
+    left -= left < kClusterMaxSteps ? left : kClusterMaxSteps;
+    ++launches;
+  }
+  while (left >= 2) {
+    int k = 1;
+    while (k < kGraphLogMax && (int64_t(2) << k) <= left) ++k;
+    const int64_t m = int64_t(1) << k;
+    launches += (h->cfg.two ? m / 2 : m) + 1;  // the steps and the epoch
+    left -= m;
+  }
+  return launches + left;
+}
+
 int64_t mclbm_steps_done(const mclbm_t* h) { return h ? h->steps : -1; }
 
 const char* mclbm_last_error(const mclbm_t* h) { return h ? h->err : "NULL handle"; }
