@@ -6,21 +6,28 @@
 // its gradients need theta' and rho'^p of the nodes next to it (the ring), which are recomputed here
 // and pull from one node further. Between two steps a CTA sends every neighbour the populations
 // that the neighbour's tile and ring pull from this tile, and nothing else: six directions of its outermost
-// line and three of the next. The populations of one node and direction travel as one word together with
-// the step's number; a word is written and read whole (64 or 128 bits), so that its number tells
-// the receiver that the values have arrived: there is no flag, no fence and no grid barrier. Two
+// line and three of the next. Three values travel as one word together with the step's number; a word
+// is written and read whole (128 bits, 64 with 16-bit storage), so that its number tells the
+// receiver that the values have arrived: there is no flag, no fence and no grid barrier. Two
 // slots per word, used in turn, are enough: a CTA writes a slot again only after it has its
 // neighbours' words of the step between, which they sent after they had read the slot.
 //
 // What bounds it: latency. A step is a chain of pulls (27 shared-memory loads), moments, collision (about
 // 250 dependent instructions) and the way of the words to L2 and back, of which the last is about 1
 // us and the rest grows with the nodes per SM. Per step, against one launch of the TMA kernel: 100 x
-// 100 1.84 us against 4.18 (cluster kernel 2.83), 128 x 128 1.90 against 4.19, with two thermal sets
-// 3.42 against 5.47, 256 x 256 2.76 against 4.36, FP16 3.18 against 4.70, 270 x 270 3.20 against 5.93.
+// 100 1.78 us against 4.18 (cluster kernel 2.83), 128 x 128 1.9 against 4.19, with two thermal sets
+// 2.63 against 5.47, 256 x 256 2.8 against 4.36, FP16 3.05 against 4.70, 276 x 276 3.3 against 5.74.
+// Two sets took 3.42 us with words of one node and direction (two words for their four values): the
+// inbox then allowed 56 tiles of 18 x 16 only. Warps of their own for the edge, so that the inner nodes
+// are done while the words are under way, took longer (128 x 128 2.75 us): the edge's own chain is
+// the step. The waits of a thread are for one word after the other, both read ahead once: what polls
+// more loads the way of the words.
 //
 // Per node the pulls, moments and collision are those of the other step kernels, and the
 // stochastic-rounding streams follow the same blocks of 2^k steps, so the states are the same bits.
 #pragma once
+
+#include <type_traits>
 
 #include "mclbm_cluster.cuh"
 
@@ -31,19 +38,9 @@ constexpr int kThreadsMax = 640;
 constexpr int kThreadsFew = 512;
 constexpr int kMinTile = 4;       // a tile's sides: an edge's two lines belong to one CTA
 constexpr int kMostAcross = 32;   // CTAs along a side: a launch has at least as many steps
-constexpr int kCorner = 5;        // words from a diagonal neighbour
+constexpr int kValues = 3;        // values of a word
 constexpr int kWordsPerThread = 2;
 constexpr int kPollLimit = 1 << 21;  // polls of a word before it is given up: seconds
-
-// A word: all stored values of one node and direction, and the step's number. FP32 with two thermal
-// sets takes two.
-template <class T, bool TWO>
-struct Word {
-  static constexpr int kValues = TWO ? 4 : 3;
-  static constexpr bool kShort = sizeof(T) == 2 && !TWO;  // 64 bits: three values, 16 of number
-  static constexpr int kBytes = kShort ? 8 : 16;
-  static constexpr int kParts = sizeof(T) == 4 && TWO ? 2 : 1;
-};
 
 __device__ __forceinline__ void store16(void* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile(
@@ -84,56 +81,55 @@ __device__ __forceinline__ void put(T* p, uint32_t v) {
   *reinterpret_cast<uint16_t*>(p) = (uint16_t)v;
 }
 
-// Sends the values v[0], v[set], ... as word w; receives them: false if the word is not there yet.
-template <class T, bool TWO>
-__device__ __forceinline__ void send(char* w, const T* v, int set, uint32_t number) {
-  using W = Word<T, TWO>;
-  const uint32_t a = bits(v), b = bits(v + set), c = bits(v + 2 * set);
-  if constexpr (W::kShort) {
-    store8(w, a | b << 16, c | number << 16);
-  } else if constexpr (sizeof(T) == 2) {
-    store16(w, a | b << 16, c | bits(v + 3 * set) << 16, 0u, number);
-  } else {
-    store16(w, a, b, c, number);
-    if constexpr (TWO) store16(w + 16, bits(v + 3 * set), 0u, 0u, number);
+// A word: three stored values and the step's number, 128 bits with FP32 storage, 64 with 16-bit.
+template <class T>
+struct Word {
+  static constexpr int kBytes = sizeof(T) == 4 ? 16 : 8;
+  using Bits = typename std::conditional<sizeof(T) == 4, uint4, uint2>::type;
+  __device__ __forceinline__ static void send(char* w, uint32_t a, uint32_t b, uint32_t c,
+                                              uint32_t number) {
+    if constexpr (sizeof(T) == 4)
+      store16(w, a, b, c, number);
+    else
+      store8(w, a | b << 16, c | number << 16);
   }
-}
-template <class T, bool TWO>
-__device__ __forceinline__ bool receive(const char* w, T* v, int set, uint32_t number) {
-  using W = Word<T, TWO>;
-  if constexpr (W::kShort) {
-    const uint2 x = load8(w);
-    if (x.y >> 16 != number) return false;
-    put(v, x.x & 0xFFFFu);
-    put(v + set, x.x >> 16);
-    put(v + 2 * set, x.y & 0xFFFFu);
-  } else if constexpr (sizeof(T) == 2) {
-    const uint4 x = load16(w);
-    if (x.w != number) return false;
-    put(v, x.x & 0xFFFFu);
-    put(v + set, x.x >> 16);
-    put(v + 2 * set, x.y & 0xFFFFu);
-    put(v + 3 * set, x.y >> 16);
-  } else {
-    const uint4 x = load16(w);
-    uint4 y = make_uint4(0u, 0u, 0u, number);
-    if constexpr (TWO) y = load16(w + 16);
-    if (x.w != number || y.w != number) return false;
-    put(v, x.x);
-    put(v + set, x.y);
-    put(v + 2 * set, x.z);
-    if constexpr (TWO) put(v + 3 * set, y.x);
+  __device__ __forceinline__ static Bits load(const char* w) {
+    if constexpr (sizeof(T) == 4)
+      return load16(w);
+    else
+      return load8(w);
   }
-  return true;
-}
+  __device__ __forceinline__ static uint32_t number(const Bits& x) {
+    if constexpr (sizeof(T) == 4)
+      return x.w;
+    else
+      return x.y >> 16;
+  }
+  __device__ __forceinline__ static uint32_t value(const Bits& x, int k) {
+    if constexpr (sizeof(T) == 4)
+      return k == 0 ? x.x : (k == 1 ? x.y : x.z);
+    else
+      return (k == 0 ? x.x : (k == 1 ? x.x >> 16 : x.y)) & 0xFFFFu;
+  }
+};
+// What a thread does with one of its words: the places of the values it sends and receives (-1: none),
+// where it sends them and where it finds them (bytes in the inbox; in < 0: no such word).
+struct Entry {
+  int from[kValues], out, to[kValues], in;
+};
 
-// How the lattice is cut: gx x gy tiles of at most bw x bh nodes. A CTA's words come from eight
-// neighbours (m = 0 .. 3: left, right, below, above; 4 .. 7: the diagonal ones), each at a fixed place.
+// How the lattice is cut: gx x gy tiles of at most bw x bh nodes, of `sets` sets of populations. A CTA's
+// words come from eight neighbours (m = 0 .. 3: left, right, below, above; 4 .. 7: the diagonal ones),
+// each at a fixed place: per node of an edge nine directions, one more for its first and its last
+// node; five from a corner.
 struct Cut {
-  int gx, gy, bw, bh;
+  int gx, gy, bw, bh, sets;
+  __host__ __device__ int per_node() const { return 9 * sets / kValues; }
+  __host__ __device__ int per_end() const { return (sets + kValues - 1) / kValues; }
+  __host__ __device__ int per_corner() const { return (5 * sets + kValues - 1) / kValues; }
   __host__ __device__ int from(int m) const {
-    const int ex = 9 * bh + 2, ey = 9 * bw + 2;
-    return m < 2 ? m * ex : (m < 4 ? 2 * ex + (m - 2) * ey : 2 * (ex + ey) + (m - 4) * kCorner);
+    const int ex = per_node() * bh + 2 * per_end(), ey = per_node() * bw + 2 * per_end();
+    return m < 2 ? m * ex : (m < 4 ? 2 * ex + (m - 2) * ey : 2 * (ex + ey) + (m - 4) * per_corner());
   }
   __host__ __device__ int words() const { return from(8); }
   __host__ __device__ int x0(int cx, int nx) const { return (int)((int64_t)cx * nx / gx); }
@@ -150,19 +146,19 @@ __host__ __device__ inline int direction(int dx, int dy) {
   if (dx == 0) return dy > 0 ? 2 : 4;
   return dy > 0 ? (dx > 0 ? 5 : 6) : (dx > 0 ? 8 : 7);
 }
-// Word r of the message from the neighbour at (sx, sy), whose edge is len nodes long: the node's lines
+// Item r of the message from the neighbour at (sx, sy), whose edge is len nodes long: the node's lines
 // beyond the edge (lx, ly: 1 or 2; 0 along the edge, where its place is `along`) and its direction.
 // From the side: per node of the edge the three directions that come in and the three along it from line
 // 1, the three that come in from line 2; and for the ring nodes at a wall, the first and the last, the
 // direction that bounces back there. From a corner: the five that reach the tile or its ring.
-__host__ __device__ inline bool word(int sx, int sy, int len, int r, int& lx, int& ly, int& along,
+__host__ __device__ inline bool item(int sx, int sy, int len, int r, int& lx, int& ly, int& along,
                                      int& q) {
   along = 0;
   if (sx != 0 && sy != 0) {
     lx = r == 3 ? 2 : 1;
     ly = r == 4 ? 2 : 1;
     q = direction(r == 1 ? 0 : -sx, r == 2 ? 0 : -sy);
-    return r < kCorner;
+    return r < 5;
   }
   const int side = sx + sy;  // in along the edge's normal, `along` the other way
   int line, in, by;
@@ -184,6 +180,61 @@ __host__ __device__ inline bool word(int sx, int sy, int len, int r, int& lx, in
   ly = sy ? line : 0;
   q = sx ? direction(in, by) : direction(by, in);
   return true;
+}
+
+// Value k of word r of that message: its item and set, false where there is none.
+__host__ __device__ inline bool value_of(const Cut& c, bool corner, int len, int r, int k, int& it,
+                                         int& set) {
+  int v = r * kValues + k, limit = 5 * c.sets;
+  it = 0;
+  if (!corner) {
+    const int group = r < c.per_node() * len ? r / c.per_node() : -1;
+    if (group >= 0) {
+      v -= group * c.per_node() * kValues;
+      limit = 9 * c.sets;
+      it = 9 * group;
+    } else {
+      const int end = (r - c.per_node() * len) / c.per_end();
+      v -= (c.per_node() * len + end * c.per_end()) * kValues;
+      limit = c.sets;
+      it = 9 * len + end;
+    }
+  }
+  it += v / c.sets;
+  set = v % c.sets;
+  return v < limit;
+}
+// Word w of CTA (cx, cy), whose tile has bw x bh nodes, of planes of `plane` places and rows of WX;
+// a word has `bytes` bytes.
+__host__ __device__ inline Entry entry_of(const Cut& c, int cx, int cy, int bw, int bh, int WX, int plane,
+                                          int bytes, int w) {
+  Entry e;
+  for (int k = 0; k < kValues; ++k) e.from[k] = e.to[k] = -1;
+  e.out = e.in = -1;
+  int m = 0;
+  while (m < 7 && w >= c.from(m + 1)) ++m;
+  const int r = w - c.from(m);
+  int sx, sy;
+  neighbour(m, sx, sy);
+  const int ox = cx + sx, oy = cy + sy;
+  if ((unsigned)ox >= (unsigned)c.gx || (unsigned)oy >= (unsigned)c.gy) return e;
+  const int len = sx ? bh : bw;  // the neighbour's edge is as long
+  for (int k = 0; k < kValues; ++k) {
+    int it, set, lx, ly, along, q;
+    if (!value_of(c, m >= 4, len, r, k, it, set)) continue;
+    if (!item(sx, sy, len, it, lx, ly, along, q)) continue;
+    const int ti = sx < 0 ? -lx : (sx > 0 ? bw - 1 + lx : along);
+    const int tj = sy < 0 ? -ly : (sy > 0 ? bh - 1 + ly : along);
+    e.to[k] = (set * kQ + q) * plane + (tj + 2) * WX + ti + 2;
+    // the same word of the message to that neighbour, for which this CTA is at (-sx, -sy)
+    item(-sx, -sy, len, it, lx, ly, along, q);
+    const int fi = sx < 0 ? lx - 1 : (sx > 0 ? bw - lx : along);
+    const int fj = sy < 0 ? ly - 1 : (sy > 0 ? bh - ly : along);
+    e.from[k] = (set * kQ + q) * plane + (fj + 2) * WX + fi + 2;
+    e.in = ((cy * c.gx + cx) * c.words() + w) * bytes;
+    e.out = ((oy * c.gx + ox) * c.words() + c.from(opposite(m)) + r) * bytes;
+  }
+  return e;
 }
 
 // Where a node's nine pulled directions come from (cluster::Sources, here places in the window).
@@ -214,8 +265,7 @@ __global__ void __launch_bounds__(MAXT, 1)
     step_resident_kernel(const StepArgs a, const Cut cut, int n, char* inbox, uint32_t* epoch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int NP = TWO ? kPlanes2 : kPlanes;
-  using W = Word<T, TWO>;
-  constexpr int kStride = W::kBytes * W::kParts;
+  using W = Word<T>;
   const Layout& L = a.L;
   const StepConsts& k = a.k;
   const int cx = (int)blockIdx.x % cut.gx, cy = (int)blockIdx.x / cut.gx;
@@ -254,42 +304,18 @@ __global__ void __launch_bounds__(MAXT, 1)
   const int at = (wj + 2) * WX + wi + 2;
   const cluster::Sources src = sources_of(L.nx, L.ny, WX, plane, i, j, there ? at : 0);
 
-  // the words this thread sends and receives
+  // the words this thread sends and receives. With one thermal set the values of a word are those of
+  // one node and direction, nine planes apart.
   const int words = cut.words();
-  char* slots = inbox + (size_t)blockIdx.x * words * kStride;
-  const size_t turn = (size_t)gridDim.x * words * kStride;
-  int from[kWordsPerThread], to[kWordsPerThread];  // places in the window, -1: none
-  char* out[kWordsPerThread];
-  const char* in[kWordsPerThread];
+  const size_t turn = (size_t)gridDim.x * words * W::kBytes;
+  Entry e[kWordsPerThread];
 #pragma unroll
   for (int x = 0; x < kWordsPerThread; ++x) {
     const int w = t + x * (int)blockDim.x;
-    from[x] = to[x] = -1;
-    out[x] = nullptr;
-    in[x] = nullptr;
-    if (w < words) {
-      int m = 0;
-      while (m < 7 && w >= cut.from(m + 1)) ++m;
-      const int r = w - cut.from(m);
-      int sx, sy, lx, ly, along, q;
-      neighbour(m, sx, sy);
-      const int nx_ = cx + sx, ny_ = cy + sy;
-      const int len = sx ? bh : bw;  // the neighbour's edge is as long
-      if ((unsigned)nx_ < (unsigned)cut.gx && (unsigned)ny_ < (unsigned)cut.gy &&
-          word(sx, sy, len, r, lx, ly, along, q)) {
-        const int ti = sx < 0 ? -lx : (sx > 0 ? bw - 1 + lx : along);
-        const int tj = sy < 0 ? -ly : (sy > 0 ? bh - 1 + ly : along);
-        to[x] = q * plane + (tj + 2) * WX + ti + 2;
-        in[x] = slots + (size_t)w * kStride;
-        // the same word of the message to that neighbour, for which this CTA is at (-sx, -sy)
-        word(-sx, -sy, len, r, lx, ly, along, q);
-        const int fi = sx < 0 ? lx - 1 : (sx > 0 ? bw - lx : along);
-        const int fj = sy < 0 ? ly - 1 : (sy > 0 ? bh - ly : along);
-        from[x] = q * plane + (fj + 2) * WX + fi + 2;
-        out[x] = inbox + ((size_t)(ny_ * cut.gx + nx_) * words + cut.from(opposite(m)) + r) * kStride;
-      }
-    }
+    e[x].in = -1;
+    if (w < words) e[x] = entry_of(cut, cx, cy, bw, bh, WX, plane, W::kBytes, w);
   }
+  auto place = [&](const int* at3, int k) { return TWO ? at3[k] : at3[0] + k * kQ * plane; };
 
   // the window's populations: the tile and what lies around it, as far as the lattice goes
   for (int e = t; e < plane; e += blockDim.x) {
@@ -350,27 +376,44 @@ __global__ void __launch_bounds__(MAXT, 1)
     __syncthreads();
     if (s + 1 < n) {
       const uint32_t number = (uint32_t)(s + 1);
-      const size_t slot = (size_t)(s & 1) * turn;
-#pragma unroll
-      for (int x = 0; x < kWordsPerThread; ++x)
-        if (from[x] >= 0) send<T, TWO>(out[x] + slot, buf + from[x], kQ * plane, number);
+      char* box = inbox + (size_t)(s & 1) * turn;
 #pragma unroll
       for (int x = 0; x < kWordsPerThread; ++x) {
-        if (to[x] < 0) continue;
-        int polls = 0;
-        while (!receive<T, TWO>(in[x] + slot, buf + to[x], kQ * plane, number)) {
-          if (++polls >= kPollLimit || *(volatile int*)&lost) {
+        if (e[x].in < 0) continue;
+        uint32_t v[kValues];
+#pragma unroll
+        for (int y = 0; y < kValues; ++y) {
+          const int p = place(e[x].from, y);
+          v[y] = !TWO || p >= 0 ? bits(buf + p) : 0u;
+        }
+        W::send(box + e[x].out, v[0], v[1], v[2], number);
+      }
+      // all words are asked for at once, then waited for one by one (without a word: the first is read)
+      typename W::Bits got[kWordsPerThread];
+#pragma unroll
+      for (int x = 0; x < kWordsPerThread; ++x) got[x] = W::load(box + max(e[x].in, 0));
+#pragma unroll
+      for (int x = 0; x < kWordsPerThread; ++x) {
+        if (e[x].in < 0) continue;
+        for (int polls = 1; W::number(got[x]) != number; ++polls) {
+          if ((polls & 255) == 0 && (polls >= kPollLimit || *(volatile int*)&lost)) {
             *(volatile int*)&lost = 1;
             atomicOr(a.err, 1);
             break;
           }
+          got[x] = W::load(box + e[x].in);
+        }
+#pragma unroll
+        for (int y = 0; y < kValues; ++y) {
+          const int p = place(e[x].to, y);
+          if (!TWO || p >= 0) put(buf + p, W::value(got[x], y));
         }
       }
       __syncthreads();
     }
   }
-  for (int e = t; e < own; e += blockDim.x) {
-    const int rr = e / bw, cc = e - rr * bw;
+  for (int u = t; u < own; u += blockDim.x) {
+    const int rr = u / bw, cc = u - rr * bw;
     T* p0 = static_cast<T*>(a.dst) + (size_t)(y0 + rr) * L.pitch + x0 + cc;
     const T* res = buf + (rr + 2) * WX + cc + 2;
 #pragma unroll
@@ -388,9 +431,7 @@ inline size_t smem_bytes(const Layout& L, const Cut& c) {
          (size_t)2 * (c.bw + 2) * (c.bh + 2) * sizeof(float);
 }
 inline size_t inbox_bytes(const Layout& L, const Cut& c) {
-  const bool two = L.np == kPlanes2;
-  const int stride = L.elem == 2 ? (two ? 16 : 8) : (two ? 32 : 16);
-  return (size_t)2 * c.gx * c.gy * c.words() * stride;
+  return (size_t)2 * c.gx * c.gy * c.words() * (L.elem == 2 ? 8 : 16);
 }
 inline int threads_of(const Cut& c) {
   const int nodes = c.bw * c.bh + 2 * (c.bw + c.bh);
@@ -433,10 +474,12 @@ cudaError_t prepare(StepConfig* c, const Layout& L, bool all, bool two) {
   int fewest = kThreadsMax + 1;
   for (int gx = 1; gx <= kMostAcross && gx * kMinTile <= L.nx; ++gx) {
     for (int gy = 1; gy <= kMostAcross && gx * gy <= sms && gy * kMinTile <= L.ny; ++gy) {
-      const Cut t{gx, gy, (L.nx + gx - 1) / gx, (L.ny + gy - 1) / gy};
-      if (threads_of(t) < fewest && smem_bytes(L, t) <= 226 * 1024 &&
+      const Cut t{gx, gy, (L.nx + gx - 1) / gx, (L.ny + gy - 1) / gy, L.np / kQ};
+      if (t.bw * t.bh >= fewest) continue;  // most cuts: too few CTAs
+      const int threads = threads_of(t);
+      if (threads < fewest && smem_bytes(L, t) <= 226 * 1024 &&
           inbox_bytes(L, t) <= (size_t)L.np * L.plane * L.elem) {
-        fewest = threads_of(t);
+        fewest = threads;
         best = t;
       }
     }
@@ -463,7 +506,7 @@ template <class T>
 cudaError_t launch(const StepArgs& a, const StepConfig& c, int n, void* scratch, uint32_t* epoch,
                    cudaStream_t st) {
   const Cut cut{c.re_gx, c.re_gy, (a.L.nx + c.re_gx - 1) / c.re_gx,
-                (a.L.ny + c.re_gy - 1) / c.re_gy};
+                (a.L.ny + c.re_gy - 1) / c.re_gy, a.L.np / kQ};
   cudaError_t e = cudaMemsetAsync(scratch, 0, inbox_bytes(a.L, cut), st);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[1];

@@ -21,8 +21,8 @@ def _built():
     (300, 7, 1, 0, 1, 127, (35, 64)),        # one CTA high, FP16 stochastic
     (37, 29, 2, 1, 1, 103, (101,)),          # BF16 to nearest, some forces off
     (110, 97, 2, 0, 1, 127, (1060, 32)),     # blocks of 1024, 32 and 4; BF16
-    (128, 128, 0, 1, 2, 127, (50, 51)),      # two thermal sets: two words per node and direction
-    (130, 131, 1, 0, 2, 127, (47,)),         # two sets, FP16: one word of four values
+    (128, 128, 0, 1, 2, 127, (50, 51)),      # two thermal sets: four values per node and direction
+    (130, 131, 1, 0, 2, 127, (47,)),         # two sets, FP16
     (256, 256, 0, 1, 1, 127, (64,)),         # tiles of 22 x 22, most threads
     (283, 241, 1, 0, 1, 127, (39,)),         # tiles of differing sizes
     (700, 64, 0, 1, 1, 126, (36,)),          # long and narrow
