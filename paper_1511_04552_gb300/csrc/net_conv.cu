@@ -17,7 +17,7 @@
 // Loss and gradient of the 256 x 256 network at batch 16: 6.33 ms with im2col rows, their GEMMs and
 // col2im, 1.58 ms with these kernels (ten forward convolutions 0.47 ms, ten weight gradients
 // 0.41 ms, nine input gradients 0.33 ms; the rest is element-wise). Forward at batch 1: 367 us (the
-// launches of 10 GEMMs with a tensor map and an occupancy query each) to 140 us.
+// launches of 10 GEMMs with a tensor map and an occupancy query each) to 120 us.
 //
 // Every mbarrier wait is bounded (2 s); a role that gives up sets the abort word, the copies and
 // MMAs in flight are drained (bounded), tensor memory is freed and the error bit is set.
