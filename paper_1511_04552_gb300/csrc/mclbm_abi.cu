@@ -377,7 +377,14 @@ int mclbm_step(mclbm_t* h, int64_t n) {
     const int64_t m = (left < kClusterMaxSteps ? left : kClusterMaxSteps) & ~int64_t(1);
     StepArgs a = step_args(h, h->cur, 0);
     a.dst = h->state[h->cur];
-    CK(h, launch_resident(a, h->cfg, (int)m, h->state[1 - h->cur], h->epoch, h->stream));
+    const cudaError_t e =
+        launch_resident(a, h->cfg, (int)m, h->state[1 - h->cur], h->epoch, h->stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {  // a stream with fewer SMs than the device
+      cudaGetLastError();
+      h->cfg.re_ctas = 0;
+      break;
+    }
+    CK(h, e);
     h->steps += m;
     left -= m;
   }

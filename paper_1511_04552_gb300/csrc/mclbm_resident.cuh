@@ -34,8 +34,8 @@
 namespace mcl {
 namespace resident {
 
-constexpr int kThreadsMax = 640;
-constexpr int kThreadsFew = 512;
+constexpr int kThreadsMax = 640;  // 96 registers each, as from 17 warps on
+constexpr int kThreadsFew = 512;  // 128: no spills
 constexpr int kMinTile = 4;       // a tile's sides: an edge's two lines belong to one CTA
 constexpr int kMostAcross = 32;   // CTAs along a side: a launch has at least as many steps
 constexpr int kValues = 3;        // values of a word
