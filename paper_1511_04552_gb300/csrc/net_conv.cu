@@ -278,8 +278,10 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_kernel(const ConvArgs a)
     }
     if (live) load();
     while (live) {
-      if (ring.round > 0 &&
-          !role_wait(smem_addr(&empty[ring.st]), (ring.round - 1) & 1u, abort)) {
+      // the warp stays or goes as one: load() votes over all its lanes
+      const bool ok = ring.round == 0 ||
+                      role_wait(smem_addr(&empty[ring.st]), (ring.round - 1) & 1u, abort);
+      if (!__all_sync(0xffffffffu, ok)) {
         *abort = 1;
         break;
       }
