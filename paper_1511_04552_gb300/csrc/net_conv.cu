@@ -387,6 +387,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_kernel(const ConvArgs a)
       const bool none = MODE == kConvPartial && it.z * a.split_steps >= a.steps;  // beyond K
 #pragma unroll 1
       for (int c0 = (warp >> 2) * 8; c0 < a.nt; c0 += 16) {
+        __syncwarp();  // lanes beyond the edge have skipped the stores of the group before
         uint32_t u[8];
         tmem_ld8_async(lane_addr + (uint32_t)c0, u);
         const int o0 = it.n * a.nt + c0;
@@ -402,32 +403,32 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_kernel(const ConvArgs a)
             beta[j] = has && f ? __ldg(f + a.N + o0 + j) : 0.f;
           }
           tmem_ld_wait();
-          if (!in) continue;
-          float out[8];
+          if (in) {
+            float out[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float pre = __uint_as_float(u[j]) + bias[j];
-            float zz = pre;
-            if (f) zz = (1.f + g[j]) * pre + beta[j];
-            u[j] = __float_as_uint(pre);
-            out[j] = e.act ? zz / (1.f + expf(-zz)) : zz;
-          }
-          if (e.pre) {
-            float* dst = e.pre + (int64_t)o0 * P + p;
+            for (int j = 0; j < 8; ++j) {
+              const float pre = __uint_as_float(u[j]) + bias[j];
+              float zz = pre;
+              if (f) zz = (1.f + g[j]) * pre + beta[j];
+              u[j] = __float_as_uint(pre);
+              out[j] = e.act ? zz / (1.f + expf(-zz)) : zz;
+            }
+            if (e.pre) {
+              float* dst = e.pre + (int64_t)o0 * P + p;
 #pragma unroll
-            for (int j = 0; j < 8; ++j, dst += P)
-              if (o0 + j < a.N) *dst = __uint_as_float(u[j]);
+              for (int j = 0; j < 8; ++j, dst += P)
+                if (o0 + j < a.N) *dst = __uint_as_float(u[j]);
+            }
+            if (e.y && o0 < a.N)
+              store_group(e, o0 / 8, it.b, y, x, a.Ho, a.Wo,
+                          make_uint4(pack2(out[0], out[1]), pack2(out[2], out[3]),
+                                     pack2(out[4], out[5]), pack2(out[6], out[7])));
           }
-          if (e.y && o0 < a.N)
-            store_group(e, o0 / 8, it.b, y, x, a.Ho, a.Wo,
-                        make_uint4(pack2(out[0], out[1]), pack2(out[2], out[3]),
-                                   pack2(out[4], out[5]), pack2(out[6], out[7])));
         } else if constexpr (MODE == kConvPartial) {
           tmem_ld_wait();
-          if (!in) continue;
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            if (o0 + j < a.N)
+            if (in && o0 + j < a.N)
               a.part[((int64_t)it.z * a.N + o0 + j) * P + p] = none ? 0.f : __uint_as_float(u[j]);
         } else {
           // channels [0, cu) to their source (2 x 2 sums, in row order, when it was upsampled),
@@ -448,18 +449,20 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_kernel(const ConvArgs a)
               v[j] += __shfl_down_sync(0xffffffffu, own, 17);
             }
           }
-          if (!in || o0 >= a.N || (up && (lane >= 16 || (lane & 1)))) continue;
-          const int64_t step = up ? P / 4 : P;
-          float* dst = first ? q.dsrc1 + (int64_t)o0 * step : q.dsrc2 + (int64_t)(o0 - q.cu) * step;
-          dst += up ? (int64_t)it.b * (hw / 4) + (y / 2) * (a.Wo / 2) + x / 2 : p;
-          if (first ? q.acc1 : q.acc2) {
+          if (in && o0 < a.N && !(up && (lane >= 16 || (lane & 1)))) {
+            const int64_t step = up ? P / 4 : P;
+            float* dst =
+                first ? q.dsrc1 + (int64_t)o0 * step : q.dsrc2 + (int64_t)(o0 - q.cu) * step;
+            dst += up ? (int64_t)it.b * (hw / 4) + (y / 2) * (a.Wo / 2) + x / 2 : p;
+            if (first ? q.acc1 : q.acc2) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) old[j] = dst[j * step];
+              for (int j = 0; j < 8; ++j) old[j] = dst[j * step];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = old[j] + v[j];
+              for (int j = 0; j < 8; ++j) v[j] = old[j] + v[j];
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) dst[j * step] = v[j];
           }
-#pragma unroll
-          for (int j = 0; j < 8; ++j) dst[j * step] = v[j];
         }
       }
       tc_fence_before();
@@ -599,6 +602,7 @@ __global__ void __launch_bounds__(kS2Threads) dx_stride2_kernel(
       const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
       for (int half = 0; half < kS2Ch / 8; ++half) {
+        __syncwarp();  // as in conv_kernel
         uint32_t d[9][8];
 #pragma unroll
         for (int tap = 0; tap < 9; ++tap)
@@ -606,28 +610,29 @@ __global__ void __launch_bounds__(kS2Threads) dx_stride2_kernel(
         tmem_ld_wait();
         auto D = [&](int tap, int j) { return __uint_as_float(d[tap][j]); };
         const int c = ch * kS2Ch + half * 8;
-        if (!in || c >= a.C) continue;  // C is a multiple of 8
-        const int64_t plane = (int64_t)a.batch * H * W;
-        float* dst = a.dsrc + (int64_t)c * plane + ((int64_t)b * H + 2 * Y) * W + 2 * X;
-        float2 top[8], bot[8];
-        if (a.accumulate) {
+        if (in && c < a.C) {  // C is a multiple of 8
+          const int64_t plane = (int64_t)a.batch * H * W;
+          float* dst = a.dsrc + (int64_t)c * plane + ((int64_t)b * H + 2 * Y) * W + 2 * X;
+          float2 top[8], bot[8];
+          if (a.accumulate) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              top[j] = *reinterpret_cast<const float2*>(dst + j * plane);
+              bot[j] = *reinterpret_cast<const float2*>(dst + j * plane + W);
+            }
+          }
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            top[j] = *reinterpret_cast<const float2*>(dst + j * plane);
-            bot[j] = *reinterpret_cast<const float2*>(dst + j * plane + W);
+            const float ee = D(4, j), eo = D(3, j) + D(5, j), oe = D(1, j) + D(7, j);
+            const float oo = ((D(0, j) + D(2, j)) + D(6, j)) + D(8, j);
+            top[j] = a.accumulate ? make_float2(top[j].x + ee, top[j].y + eo) : make_float2(ee, eo);
+            bot[j] = a.accumulate ? make_float2(bot[j].x + oe, bot[j].y + oo) : make_float2(oe, oo);
           }
-        }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const float ee = D(4, j), eo = D(3, j) + D(5, j), oe = D(1, j) + D(7, j);
-          const float oo = ((D(0, j) + D(2, j)) + D(6, j)) + D(8, j);
-          top[j] = a.accumulate ? make_float2(top[j].x + ee, top[j].y + eo) : make_float2(ee, eo);
-          bot[j] = a.accumulate ? make_float2(bot[j].x + oe, bot[j].y + oo) : make_float2(oe, oo);
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          *reinterpret_cast<float2*>(dst + j * plane) = top[j];
-          *reinterpret_cast<float2*>(dst + j * plane + W) = bot[j];
+          for (int j = 0; j < 8; ++j) {
+            *reinterpret_cast<float2*>(dst + j * plane) = top[j];
+            *reinterpret_cast<float2*>(dst + j * plane + W) = bot[j];
+          }
         }
       }
       tc_fence_before();

@@ -44,3 +44,23 @@ def test_waits_before_a_vote_are_voted_on(name):
         alone = re.search(r"if \([^;{]*!(?:role|cluster)_wait\(", role)
         assert not alone, role[alone.start():alone.end() + 80]
     assert seen >= 2
+
+
+@pytest.mark.parametrize("name", ["net_conv.cu", "net_gemm.cu"])
+def test_lanes_meet_before_tensor_memory_loads(name):
+    """tcgen05.ld is undefined unless all 32 lanes execute it together: in a loop around one no lane
+    goes on alone, and the lanes meet before the load (tmem_ld16 does that itself)."""
+    src = _source(name)
+    helper, _ = _block(_source("net_tc.cuh"), _source("net_tc.cuh").index("void tmem_ld16("))
+    assert helper.index("__syncwarp();") < helper.index("tcgen05.ld")
+    seen = 0
+    for m in re.finditer(r"\bfor \([^{}]*?\) \{", src):
+        body, _ = _block(src, m.end() - 1)
+        inner = min((body.find(t) for t in ("tmem_ld16(", "tmem_ld8_async(") if t in body), default=-1)
+        if inner < 0 or "role_wait(" in body or "cluster_wait(" in body or "bar_wait(" in body:
+            continue  # none, or a loop over tiles, whose waits are voted on
+        seen += 1
+        assert "continue;" not in body, body[:200]
+        if "tmem_ld8_async(" in body:
+            assert 0 <= body.find("__syncwarp();") < inner, body[:200]
+    assert seen >= 2
