@@ -63,6 +63,15 @@ int64_t resident_min_steps(const StepConfig& c) {
   return across <= 16 ? 16 : (across + 1) & ~1;
 }
 
+// A resident kernel's launch that is refused because its CTAs cannot all be placed at once (a stream with
+// fewer SMs than the device, as of a green context): nothing has run, and the handle goes on with the
+// step-by-step kernels, which need no CTA beside another. Any other error is the caller's.
+bool not_placeable(cudaError_t e) {
+  return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize ||
+         e == cudaErrorInvalidConfiguration || e == cudaErrorLaunchOutOfResources ||
+         e == cudaErrorInvalidResourceConfiguration;
+}
+
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 int fail(mclbm_t* h, int code, const char* fmt, ...) {
@@ -312,7 +321,7 @@ int mclbm_bind(mclbm_t* h, void* dev_buf, size_t bytes, void* cuda_stream) {
   if ((!sv || std::strcmp(sv, "cluster") == 0) && !std::getenv("MCLBM_STEP_VEC") &&
       !std::getenv("MCLBM_STEP_TILE_H") &&
       prepare_cluster(&h->cfg, h->L, h->k.mask == MCLBM_F_ALL && !h->k.two_sets,
-                      h->k.two_sets != 0) != cudaSuccess) {
+                      h->k.two_sets != 0, h->stream) != cudaSuccess) {
     cudaGetLastError();
     h->cfg.cl_ctas = 0;
   }
@@ -379,7 +388,7 @@ int mclbm_step(mclbm_t* h, int64_t n) {
     a.dst = h->state[h->cur];
     const cudaError_t e =
         launch_resident(a, h->cfg, (int)m, h->state[1 - h->cur], h->epoch, h->stream);
-    if (e == cudaErrorCooperativeLaunchTooLarge) {  // a stream with fewer SMs than the device
+    if (not_placeable(e)) {
       cudaGetLastError();
       h->cfg.re_ctas = 0;
       break;
@@ -394,7 +403,14 @@ int mclbm_step(mclbm_t* h, int64_t n) {
     StepArgs a = step_args(h, h->cur, 0);
     const int to = h->cur ^ (int)(m & 1);
     a.dst = h->state[to];
-    CK(h, launch_cluster(a, h->cfg, (int)m, (uint32_t)h->steps, h->epoch, h->stream));
+    const cudaError_t e =
+        launch_cluster(a, h->cfg, (int)m, (uint32_t)h->steps, h->epoch, h->stream);
+    if (not_placeable(e)) {
+      cudaGetLastError();
+      h->cfg.cl_ctas = 0;
+      break;
+    }
+    CK(h, e);
     h->cur = to;
     h->steps += m;
     left -= m;

@@ -299,9 +299,9 @@ inline void fill_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, cons
 }
 
 // Sets c.cl_* where the kernel is to run (CTAs 0: it is not): a run's nodes fit the threads, its
-// populations shared memory, and the device can place the cluster.
+// populations shared memory, and the SMs that the stream may use can hold the cluster.
 template <class T>
-cudaError_t prepare(StepConfig* c, const Layout& L, bool all, bool two) {
+cudaError_t prepare(StepConfig* c, const Layout& L, bool all, bool two, cudaStream_t st) {
   c->cl_ctas = 0;
   const int64_t nodes = (int64_t)L.nx * L.ny;
   const int line = std::min(L.nx, L.ny);
@@ -325,7 +325,7 @@ cudaError_t prepare(StepConfig* c, const Layout& L, bool all, bool two) {
       return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = {};
-    fill_config(&cfg, attr, t, L, nullptr);
+    fill_config(&cfg, attr, t, L, st);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n >= 1) {
       *c = t;

@@ -110,14 +110,17 @@ cudaError_t make_two_step_tensor_map(CUtensorMap* map, void* state0, const Layou
 cudaError_t prepare_two_f32(StepConfig* c, const Layout& L);
 cudaError_t launch_two_f32(const StepArgs& a, const StepConfig& c, const CUtensorMap* map2,
                            cudaStream_t st);
-// Cluster-resident kernel: enables it in c where the lattice fits one cluster; n steps in one launch
-// from a.src to a.dst.
-cudaError_t prepare_cluster(StepConfig* c, const Layout& L, bool all, bool two);
+// Cluster-resident kernel: enables it in c where the lattice fits one cluster that the stream's SMs can
+// hold; n steps in one launch from a.src to a.dst.
+cudaError_t prepare_cluster(StepConfig* c, const Layout& L, bool all, bool two, cudaStream_t st);
 cudaError_t launch_cluster(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
                            uint32_t* epoch, cudaStream_t st);
-cudaError_t prepare_cluster_f32(StepConfig* c, const Layout& L, bool all, bool two);
-cudaError_t prepare_cluster_f16(StepConfig* c, const Layout& L, bool all, bool two);
-cudaError_t prepare_cluster_bf16(StepConfig* c, const Layout& L, bool all, bool two);
+cudaError_t prepare_cluster_f32(StepConfig* c, const Layout& L, bool all, bool two,
+                                cudaStream_t st);
+cudaError_t prepare_cluster_f16(StepConfig* c, const Layout& L, bool all, bool two,
+                                cudaStream_t st);
+cudaError_t prepare_cluster_bf16(StepConfig* c, const Layout& L, bool all, bool two,
+                                cudaStream_t st);
 cudaError_t launch_cluster_f32(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
                                uint32_t* epoch, cudaStream_t st);
 cudaError_t launch_cluster_f16(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,

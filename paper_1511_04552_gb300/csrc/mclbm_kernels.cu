@@ -500,14 +500,14 @@ cudaError_t launch_step(const StepArgs& a, const StepConfig& c, const CUtensorMa
   }
 }
 
-cudaError_t prepare_cluster(StepConfig* c, const Layout& L, bool all, bool two) {
+cudaError_t prepare_cluster(StepConfig* c, const Layout& L, bool all, bool two, cudaStream_t st) {
   switch (L.storage) {
     case MCLBM_STORE_F32:
-      return prepare_cluster_f32(c, L, all, two);
+      return prepare_cluster_f32(c, L, all, two, st);
     case MCLBM_STORE_F16:
-      return prepare_cluster_f16(c, L, all, two);
+      return prepare_cluster_f16(c, L, all, two, st);
     case MCLBM_STORE_BF16:
-      return prepare_cluster_bf16(c, L, all, two);
+      return prepare_cluster_bf16(c, L, all, two, st);
     default:
       return cudaErrorInvalidValue;
   }

@@ -17,8 +17,9 @@ cudaError_t prepare_tma_f16(StepConfig* c, const Layout& L) {
   return pair::prepare_pair_tma_t<__half>(c, L);
 }
 
-cudaError_t prepare_cluster_f16(StepConfig* c, const Layout& L, bool all, bool two) {
-  return cluster::prepare<__half>(c, L, all, two);
+cudaError_t prepare_cluster_f16(StepConfig* c, const Layout& L, bool all, bool two,
+                                cudaStream_t st) {
+  return cluster::prepare<__half>(c, L, all, two, st);
 }
 
 cudaError_t launch_cluster_f16(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,

@@ -25,8 +25,9 @@ cudaError_t launch_two_f32(const StepArgs& a, const StepConfig& c, const CUtenso
   return pair::launch_two(a, c, map2, st);
 }
 
-cudaError_t prepare_cluster_f32(StepConfig* c, const Layout& L, bool all, bool two) {
-  return cluster::prepare<float>(c, L, all, two);
+cudaError_t prepare_cluster_f32(StepConfig* c, const Layout& L, bool all, bool two,
+                                cudaStream_t st) {
+  return cluster::prepare<float>(c, L, all, two, st);
 }
 
 cudaError_t launch_cluster_f32(const StepArgs& a, const StepConfig& c, int n, uint32_t steps0,
