@@ -6,8 +6,8 @@
 // its gradients need theta' and rho'^p of the nodes next to it (the ring), which are recomputed here
 // and pull from one node further. Between two steps a CTA sends every neighbour the populations
 // that the neighbour's tile and ring pull from this tile, and nothing else: six directions of its outermost
-// line and three of the next. Three values travel as one word together with the step's number; a word
-// is written and read whole (128 bits, 64 with 16-bit storage), so that its number tells the
+// line and three of the next. Three values travel as one word together with the step's mark; a word
+// is written and read whole (128 bits, 64 with 16-bit storage), so that its mark tells the
 // receiver that the values have arrived: there is no flag, no fence and no grid barrier. Two
 // slots per word, used in turn, are enough: a CTA writes a slot again only after it has its
 // neighbours' words of the step between, which they sent after they had read the slot.
@@ -81,17 +81,27 @@ __device__ __forceinline__ void put(T* p, uint32_t v) {
   *reinterpret_cast<uint16_t*>(p) = (uint16_t)v;
 }
 
-// A word: three stored values and the step's number, 128 bits with FP32 storage, 64 with 16-bit.
+// A word: three stored values and their exclusive or with the step's mark, 128 bits with FP32 storage, 64
+// with 16-bit. The poll's test takes every lane of the word: a relaxed 128-bit load proved whole only where
+// all its lanes are used. Words of one value, with a number in the last lane and two lanes that nobody read, of
+// which the poll tested the number and the value was used after it, came with the new number and the old value
+// (FP32, two thermal sets: every run of 16 steps was off); with those two lanes tested as well, none did.
 template <class T>
 struct Word {
   static constexpr int kBytes = sizeof(T) == 4 ? 16 : 8;
   using Bits = typename std::conditional<sizeof(T) == 4, uint4, uint2>::type;
+  // The mark of step number 1 .. 2^14: not 0, as in the inbox before the first step, and its neighbours
+  // differ in many bits, so that old and new values a few bits apart don't make up for it.
+  __device__ __forceinline__ static uint32_t mark(uint32_t number) {
+    return sizeof(T) == 4 ? number * 0x9E3779B1u : number * 0x9E37u & 0xFFFFu;
+  }
   __device__ __forceinline__ static void send(char* w, uint32_t a, uint32_t b, uint32_t c,
-                                              uint32_t number) {
+                                              uint32_t mark) {
+    const uint32_t d = a ^ b ^ c ^ mark;
     if constexpr (sizeof(T) == 4)
-      store16(w, a, b, c, number);
+      store16(w, a, b, c, d);
     else
-      store8(w, a | b << 16, c | number << 16);
+      store8(w, a | b << 16, c | d << 16);
   }
   __device__ __forceinline__ static Bits load(const char* w) {
     if constexpr (sizeof(T) == 4)
@@ -99,11 +109,13 @@ struct Word {
     else
       return load8(w);
   }
-  __device__ __forceinline__ static uint32_t number(const Bits& x) {
-    if constexpr (sizeof(T) == 4)
-      return x.w;
-    else
-      return x.y >> 16;
+  __device__ __forceinline__ static bool is(const Bits& x, uint32_t mark) {
+    if constexpr (sizeof(T) == 4) {
+      return (x.x ^ x.y ^ x.z ^ x.w) == mark;
+    } else {
+      const uint32_t both = x.x ^ x.y;
+      return ((both ^ both >> 16) & 0xFFFFu) == mark;
+    }
   }
   __device__ __forceinline__ static uint32_t value(const Bits& x, int k) {
     if constexpr (sizeof(T) == 4)
@@ -258,8 +270,8 @@ __device__ __forceinline__ cluster::Sources sources_of(int nx, int ny, int WX, i
   return s;
 }
 
-// n steps (even) from a.src to a.dst, the same level; steps0: steps done before this launch. inbox: two
-// slots for every word of every CTA, zero at the start.
+// n steps (even) from a.src to a.dst, the same level. inbox: two slots for every word of every CTA, zero
+// at the start.
 template <class T, bool SR, bool ALLF, bool TWO, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1)
     step_resident_kernel(const StepArgs a, const Cut cut, int n, char* inbox, uint32_t* epoch) {
@@ -375,7 +387,7 @@ __global__ void __launch_bounds__(MAXT, 1)
     }
     __syncthreads();
     if (s + 1 < n) {
-      const uint32_t number = (uint32_t)(s + 1);
+      const uint32_t mark = W::mark((uint32_t)(s + 1));
       char* box = inbox + (size_t)(s & 1) * turn;
 #pragma unroll
       for (int x = 0; x < kWordsPerThread; ++x) {
@@ -386,7 +398,7 @@ __global__ void __launch_bounds__(MAXT, 1)
           const int p = place(e[x].from, y);
           v[y] = !TWO || p >= 0 ? bits(buf + p) : 0u;
         }
-        W::send(box + e[x].out, v[0], v[1], v[2], number);
+        W::send(box + e[x].out, v[0], v[1], v[2], mark);
       }
       // all words are asked for at once, then waited for one by one (without a word: the first is read)
       typename W::Bits got[kWordsPerThread];
@@ -395,7 +407,7 @@ __global__ void __launch_bounds__(MAXT, 1)
 #pragma unroll
       for (int x = 0; x < kWordsPerThread; ++x) {
         if (e[x].in < 0) continue;
-        for (int polls = 1; W::number(got[x]) != number; ++polls) {
+        for (int polls = 1; !W::is(got[x], mark); ++polls) {
           if ((polls & 255) == 0 && (polls >= kPollLimit || *(volatile int*)&lost)) {
             *(volatile int*)&lost = 1;
             atomicOr(a.err, 1);
