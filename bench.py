@@ -34,16 +34,16 @@ UNIT = "MLUPS"
 BYTES_PER_LU = 216  # 27 FP32 populations read + 27 written per lattice-node update
 STORAGE = {"f32": (0, 216), "f16": (1, 108), "bf16": (2, 108)}  # (code, bytes per update)
 CHUNK = 1000        # time steps per benchmark step (one residual / Nusselt check interval)
-OUR_KERNELS_PER_REDUCTION = 5  # nusselt, residual + final, mass + final
+RESIDENT_STEPS = 1 << 14  # most steps of one launch of a resident kernel
 WORKLOADS = {"cavity256": workloads.CAVITY_256, "cavity1024": workloads.CAVITY_1024}
 STEP_SOURCES = ("mclbm_device.cuh", "mclbm_pair.cuh")  # the step kernels' source
 
 
 def step_launches(n):
     """Kernel launches of mclbm_step(n) on a cavity that does not fit shared memory (the library's
-    decomposition; mclbm_step_launches counts for a given cavity): the even part in graphs of
-    2^k <= 1024 steps, largest first, each graph one step kernel per step and one epoch kernel;
-    an odd last step as a single launch."""
+    decomposition; mclbm_step_launches counts for a given cavity, and fewer where a resident kernel
+    runs): the even part in graphs of 2^k <= 1024 steps, largest first, each graph one step kernel
+    per step and one epoch kernel; an odd last step as a single launch."""
     launches, left = 0, n
     while left >= 2:
         k = 1
@@ -59,6 +59,35 @@ def nodes_per_thread(nx, ny, sms):
     every SM at most two 32 x 8 tiles, two beyond."""
     tiles = ((nx + 31) // 32) * ((ny + 7) // 8)
     return 1 if tiles <= 2 * sms else 2
+
+
+def reduction_launches(ny):
+    """Kernels of the Nusselt numbers, the residual and the masses: the last two with a final sum, the
+    first too where the walls are longer than one block walks (256 rows)."""
+    return 5 if ny <= 256 else 6
+
+
+def step_roofline(cav, n, step_time, state_bytes, hbm_peak, peak_kind, traffic, nodes):
+    """What bounds a step of cav.step(n) that takes step_time seconds, where one step's state read and
+    written is state_bytes. One launch per step moves the state through memory; a resident kernel
+    (mclbm_step_launches counts fewer launches than steps) does so once per launch, and its steps wait
+    for each other. The cluster kernel takes odd numbers of steps, the grid-resident one leaves the last
+    to a launch of its own."""
+    line = {"peak": hbm_peak, "unit": "GB/s", "peak_kind": peak_kind}
+    if cav.step_launches(n) < step_launches(n):
+        cluster = cav.step_launches(65) == 1
+        per = min(n, RESIDENT_STEPS) if cluster else min(n, RESIDENT_STEPS) & ~1
+        line.update(bound="latency", traffic=None, steps_per_launch=per,
+                    kernel="step_cluster_kernel" if cluster else "step_resident_kernel",
+                    nodes_per_thread=1)
+    else:
+        line.update(bound="hbm", traffic=traffic, steps_per_launch=1, kernel="step_pair_tma_kernel",
+                    nodes_per_thread=nodes)
+    line["launch_us"] = step_time * 1e6 * line["steps_per_launch"]
+    line["bytes_per_launch"] = state_bytes
+    line["achieved"] = state_bytes / line["launch_us"] / 1e3
+    line["frac"] = line["achieved"] / hbm_peak
+    return line
 
 
 def parse():
@@ -437,9 +466,7 @@ def main():
     value = whole_job_rate(lu, ws, elapsed)
     hbm_peak, peak_kind = peaks()
     sms = torch.cuda.get_device_properties(local).multi_processor_count
-    achieved = bytes_lu * nx * ny / step_time / 1e9
     launches = cav.step_launches(CH)
-    per_launch = CH if launches < CH else 1  # steps of one launch (all: state in shared memory)
 
     # end to end through the C ABI with host buffers: H2D warm fields, init, 1000 steps,
     # all 8 fields and the Nusselt numbers back to the host
@@ -502,21 +529,13 @@ def main():
                        "parallelism": "replicas" if ws > 1 else "single",
                        "l2": "flushed between bench steps (256 MiB write); state %.0f MB" % (
                            2 * 27 * 4 * nx * ny / 1e6)},
-            "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
-                         "frac": achieved / hbm_peak,
-                         "traffic": ncu_traffic(w["name"])
-                                    if args.storage == "f32" and per_launch == 1 else None,
-                         "peak_kind": peak_kind,
-                         "kernel": "step_pair_tma_kernel" if per_launch == 1 else
-                                   "step_resident_kernel",
-                         "nodes_per_thread": nodes_per_thread(nx, ny, sms),
-                         "steps_per_launch": per_launch,
-                         "bytes_per_launch": bytes_lu * nx * ny * per_launch,
-                         "launch_us": step_time * 1e6 * per_launch},
+            "roofline": step_roofline(cav, CH, step_time, bytes_lu * nx * ny, hbm_peak, peak_kind,
+                                      ncu_traffic(w["name"]) if args.storage == "f32" else None,
+                                      nodes_per_thread(nx, ny, sms)),
             "e2e": {"value": e2e_value, "unit": UNIT,
                     "h2d_bytes_per_step": 4 * nx * ny * 4,
                     "d2h_bytes_per_step": 8 * nx * ny * 4 + 16},
-            "gpu_launches": args.steps * (launches + OUR_KERNELS_PER_REDUCTION),
+            "gpu_launches": args.steps * (launches + reduction_launches(ny)),
             "clocks": clk.summary(),
         }
         line.update(extras)
