@@ -160,13 +160,17 @@ int mclbm_init(mclbm_t *h, int mode, const float *warm_dev);
 
 /* Advances n >= 0 time steps (Eqs 18-19 with the forces of Table 1 and the walls of
  * Eqs 34-36). Lattices of up to about 75 000 nodes run a call of several steps in one launch (up to
- * 2^14 steps each), the cavity resident in shared memory: the small ones in one thread-block cluster,
- * the larger ones (from 16 steps) in a cooperative grid over the device, which uses the state level
- * that is not current as scratch; others run the even part in captured CUDA graphs of 2^k steps (2 <= 2^k <= 1024, largest first, built on
- * first use and kept with the handle) and an odd last step as a single launch, with the same states
- * bit for bit. The stochastic-rounding streams of 16-bit storage follow the graphs' replay count, so a given
- * sequence of calls is reproducible bit for bit. Async. A step kernel
- * that gives up a bounded wait on its own data movement sets an error word instead of
+ * 2^14 steps each), the cavity resident in shared memory: the small ones in one thread-block
+ * cluster, the larger ones (from 16 steps) in a cooperative grid over the device, which uses the
+ * state level that is not current as scratch. Others, and a handle whose stream cannot hold the
+ * cluster or the grid, run the even part in captured CUDA graphs of 2^k steps (2 <= 2^k <= 1024,
+ * largest first, built on first use and kept with the handle) and an odd last step as a single
+ * launch, with the same states bit for bit. The grid takes every SM: cavities of about 100 x 100 to
+ * 200 x 200 that are stepped at once on streams of their own run one or two at a time, which from four
+ * (two thermal sets, 180 x 180) or eight (100 x 100, 128 x 128) on takes longer than the step-by-step
+ * kernels side by side; batch them (mclbm_batch_step) or bind them with MCLBM_STEP_VARIANT=tma in
+ * the environment. The stochastic-rounding streams of 16-bit storage follow the graphs' replay
+ * count, so a given sequence of calls is reproducible bit for bit. Async. A step kernel that gives up a bounded wait on its own data movement sets an error word instead of
  * hanging; the next mclbm_nusselt, mclbm_mass or mclbm_residual returns MCLBM_ETIMEOUT. */
 int mclbm_step(mclbm_t *h, int64_t n);
 

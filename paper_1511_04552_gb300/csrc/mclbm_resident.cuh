@@ -12,16 +12,26 @@
 // slots per word, used in turn, are enough: a CTA writes a slot again only after it has its
 // neighbours' words of the step between, which they sent after they had read the slot.
 //
-// What bounds it: latency. A step is a chain of pulls (27 shared-memory loads), moments, collision (about
-// 250 dependent instructions) and the way of the words to L2 and back, of which the last is about 1
-// us and the rest grows with the nodes per SM. Per step, against one launch of the TMA kernel: 100 x
-// 100 1.78 us against 4.18 (cluster kernel 2.83), 128 x 128 1.9 against 4.19, with two thermal sets
-// 2.63 against 5.47, 256 x 256 2.8 against 4.36, FP16 3.05 against 4.70, 276 x 276 3.3 against 5.74.
+// What bounds it: latency. A step is a chain of pulls (27 shared-memory loads), moments, collision
+// (about 250 dependent instructions) and the way of the words to L2 and back, of which the last is about
+// 1 us and the rest grows with the nodes per SM. Per step, against one launch of the TMA kernel: 100 x
+// 100 1.77 us against 4.18 (cluster kernel 2.83), 128 x 128 1.98 against 4.19, with two thermal sets
+// 2.64 against 5.47, 256 x 256 2.85 against 4.36, FP16 3.12 against 4.70, 276 x 276 3.3 against 5.74.
 // Two sets took 3.42 us with words of one node and direction (two words for their four values): the
 // inbox then allowed 56 tiles of 18 x 16 only. Warps of their own for the edge, so that the inner nodes
-// are done while the words are under way, took longer (128 x 128 2.75 us): the edge's own chain is
-// the step. The waits of a thread are for one word after the other, both read ahead once: what polls
-// more loads the way of the words.
+// are done while the words are under way, took longer (128 x 128 2.75 us): the edge's own chain is the
+// step. The waits of a thread are for one word after the other, both read ahead once: what polls more
+// loads the way of the words.
+//
+// What it gives up is other cavities beside it: the latency leaves issue slots that a second grid could
+// use, but at 128 registers only small CTAs share an SM. Several cavities stepped at once, each on a
+// stream of its own, per step and cavity with 1, 4 and 8 of them, against the TMA or tile kernel: 100 x
+// 100 1.77, 0.69, 0.69 against 4.09, 1.04, 0.58; 128 x 128 1.98, 1.09, 1.10 against 4.16, 1.07, 0.72;
+// with two sets 2.64, 2.58, 2.57 against 5.38, 1.45, 1.00; 180 x 180 2.14, 2.13, 2.13 against 4.45,
+// 1.54, 1.54; 256 x 256 gains at any number. Bounds of two CTAs of 352 threads per SM (88 registers,
+// spills) give 0.55, 0.78, 1.44 and 1.48 with eight, but take 11 to 17 % longer for one: the launch
+// bounds keep to one cavity; who steps many of these sizes at once batches them (mclbm_batch_step) or
+// asks for the other kernels (MCLBM_STEP_VARIANT).
 //
 // Per node the pulls, moments and collision are those of the other step kernels, and the
 // stochastic-rounding streams follow the same blocks of 2^k steps, so the states are the same bits.
@@ -40,7 +50,7 @@ constexpr int kMinTile = 4;       // a tile's sides: an edge's two lines belong 
 constexpr int kMostAcross = 32;   // CTAs along a side: a launch has at least as many steps
 constexpr int kValues = 3;        // values of a word
 constexpr int kWordsPerThread = 2;
-constexpr int kPollLimit = 1 << 21;  // polls of a word before it is given up: seconds
+constexpr int kPollLimit = 1 << 21;  // polls of a word before it is given up: a third of a second at least
 
 __device__ __forceinline__ void store16(void* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile(

@@ -1,6 +1,6 @@
 // C ABI of the warm-start network (include/mclbm_net.h): workspace planning, the forward and
 // backward sequences of launches, Adam, and the exposed tensor-core GEMM. Host code only; the
-// kernels are in net_gemm.cu and net_kernels.cu.
+// kernels are in net_conv.cu, net_kernels.cu and net_gemm.cu.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -573,7 +573,7 @@ int finish(mclbm_net* n, double* loss) {
     e = cudaMemcpyAsync(&l, n->loss, sizeof(double), cudaMemcpyDeviceToHost, n->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(n->stream);
   if (e != cudaSuccess) return cuda_fail(n, e, "mclbm_net sync");
-  if (err) return fail(n, MCLBM_ETIMEOUT, "a tensor-core GEMM gave up a bounded wait");
+  if (err) return fail(n, MCLBM_ETIMEOUT, "a tensor-core kernel gave up a bounded wait");
   if (loss) {
     *loss = l;
     if (!std::isfinite(l)) return fail(n, MCLBM_EDIVERGED, "loss is not finite");

@@ -34,8 +34,8 @@ struct GemmArgs {
   int splits;  // set by launch_gemm: K splits (tiles of D are m x n x split)
 };
 
-// Checks the operand requirements and launches a persistent grid over the ceil(M/128) x
-// ceil(N/128) x splits tiles of D.
+// Checks the operand requirements and launches a persistent grid over the tiles of D and the K
+// splits: 256 x 256 tiles by pairs of CTAs where that pays (pair_pays), else 128 x 128.
 cudaError_t launch_gemm(const GemmArgs& g, int splits, cudaStream_t st);
 // True if the arguments satisfy the alignment and extent rules of launch_gemm.
 bool gemm_args_valid(const GemmArgs& g, int splits);
